@@ -15,15 +15,17 @@
 // zero ghost, source scaling and trilinear points as in the isotropic path;
 // the source enters both fields, receivers interpolate p.
 //
-// Step kernel (2.5D, one point per thread, a CTA owning a 32 x 8 xy tile and
-// a run of z planes; k_tti_q, fd_tti_q.cuh): each plane of p and q enters
-// once, by TMA, with an R-wide halo; its in-plane second derivatives and its
-// first x and y differences are formed then, and every z sum (D_zz, D_xz,
-// D_yz) runs over per-thread register queues, so shared memory holds only
-// the entering plane, one plane of first x differences and the update's
-// per-point tiles.  The model enters through six per-cell fields
+// Step kernel (2.5D, one point per thread, a CTA owning a 32-wide xy tile and
+// a run of z planes; k_tti_q, fd_tti_q.cuh): p and q are stored interleaved,
+// one float2 per cell, and run through the stencil as packed pairs.  Each
+// plane enters once, by TMA, with an R-wide halo; its in-plane second
+// derivatives and its first x and y differences are formed then, and every z
+// sum (D_zz, D_xz, D_yz) runs over per-thread register queues, so shared
+// memory holds only the entering plane, one plane of first y differences and
+// the update's per-point tiles.  The model enters through six per-cell fields
 // (dt^2 v^2 / h^2, 1 + 2 eps, sqrt(1 + 2 delta) and the axis n), computed
-// once per model in double precision.
+// once per model in double precision.  fd_tti_set_state and fd_tti_get_state
+// convert between the caller's separate p and q arrays and the pairs.
 #include <math.h>
 #include <string.h>
 
@@ -50,9 +52,10 @@ struct fd_tti_s {
   size_t ncell = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  float* p[2] = {nullptr, nullptr};  // p[cur] = p^n, p[cur^1] = p^{n-1}
-  float* q[2] = {nullptr, nullptr};
-  float* coef = nullptr;  // six padded fields: A, e2, dl, nx, ny, nz
+  float2* u[2] = {nullptr, nullptr};  // (p, q): u[cur] at t_n, u[cur^1] at t_{n-1}
+  // model on the padded grid: pairs (A, e2), (dl, nz), (nx, ny), field f at
+  // coef + f * ncell
+  float2* coef = nullptr;
   int cur = 0;
   bool model_set = false;
   double vmax = 0.0, cfl = 0.0;
@@ -61,8 +64,9 @@ struct fd_tti_s {
   DevBuf inj, rec, stage_val, stage_rec, stage_in, scratch;
   DevBuf err;  // error word of the TMA kernel's bounded waits
   // tensor maps of the step kernel, per buffer
-  CUtensorMap halo_p[2], halo_q[2], tile_p[2], tile_q[2], coef_map;
+  CUtensorMap halo[2], tile[2], coef_map;
   long long spin_limit = 0;
+  int ctas = 0;  // persistent CTAs of a step (0: not known yet)
   int n_inj = 0, n_rec = 0;
   bool profiling = false;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -71,6 +75,8 @@ struct fd_tti_s {
 };
 
 namespace {
+
+constexpr size_t kStageBytes = size_t(32) << 20;  // staging of host states
 
 struct TtiInj {
   long long off;
@@ -98,13 +104,13 @@ __global__ void k_tti_coef(const float* __restrict__ vp, const float* __restrict
                            const float* __restrict__ del, const float* __restrict__ th,
                            const float* __restrict__ ph, int nx, int ny, int nz, int nbl,
                            int Nx, int Ny, int pitch, size_t ncell, double dt2_h2,
-                           float* __restrict__ coef) {
+                           float2* __restrict__ coef) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y, z = blockIdx.z;
   if (x >= pitch) return;
   const size_t o = (static_cast<size_t>(z) * Ny + y) * pitch + x;
   if (x >= Nx) {
-    for (int f = 0; f < 6; ++f) coef[f * ncell + o] = 0.f;
+    for (int f = 0; f < 3; ++f) coef[f * ncell + o] = make_float2(0.f, 0.f);
     return;
   }
   const int px = min(max(x - nbl, 0), nx - 1);
@@ -112,12 +118,13 @@ __global__ void k_tti_coef(const float* __restrict__ vp, const float* __restrict
   const int pz = min(max(z - nbl, 0), nz - 1);
   const size_t i = (static_cast<size_t>(pz) * ny + py) * nx + px;
   const double v = vp[i], t = th[i], p = ph[i];
-  coef[o] = static_cast<float>(dt2_h2 * v * v);
-  coef[ncell + o] = static_cast<float>(1.0 + 2.0 * static_cast<double>(eps[i]));
-  coef[2 * ncell + o] = static_cast<float>(sqrt(1.0 + 2.0 * static_cast<double>(del[i])));
-  coef[3 * ncell + o] = static_cast<float>(sin(t) * cos(p));
-  coef[4 * ncell + o] = static_cast<float>(sin(t) * sin(p));
-  coef[5 * ncell + o] = static_cast<float>(cos(t));
+  coef[o] = make_float2(static_cast<float>(dt2_h2 * v * v),
+                        static_cast<float>(1.0 + 2.0 * static_cast<double>(eps[i])));
+  coef[ncell + o] =
+      make_float2(static_cast<float>(sqrt(1.0 + 2.0 * static_cast<double>(del[i]))),
+                  static_cast<float>(cos(t)));
+  coef[2 * ncell + o] =
+      make_float2(static_cast<float>(sin(t) * cos(p)), static_cast<float>(sin(t) * sin(p)));
 }
 
 // max of v sqrt(1+2 eps) (bits of a non-negative float) and the count of
@@ -149,60 +156,82 @@ __global__ void k_tti_stats(const float* __restrict__ vp, const float* __restric
 }
 
 // rec[row][r] = sum_k w_k p[off_k]
-__global__ void k_tti_gather(const float* __restrict__ p, const TtiRec* __restrict__ recs, int n,
+__global__ void k_tti_gather(const float2* __restrict__ u, const TtiRec* __restrict__ recs, int n,
                              float* __restrict__ out) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   const TtiRec e = recs[r];
   float acc = 0.f;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc = fmaf(e.w[k], p[e.off[k]], acc);
+  for (int k = 0; k < 8; ++k) acc = fmaf(e.w[k], u[e.off[k]].x, acc);
   out[r] = acc;
 }
 
 // p, q at each source node += A w q(t_n) / (h (1 + b)) (s^n = w q / h^3 scaled
 // by dt^2 v^2 and the damping division of the update)
 __global__ void k_tti_inject(const TtiInj* __restrict__ inj, int n, const float* __restrict__ val,
-                             const float* __restrict__ A, float bscale, int nbl, int nx, int ny,
-                             int nz, float* p, float* q) {
+                             const float2* __restrict__ coef, float bscale, int nbl, int nx, int ny,
+                             int nz, float2* u) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const TtiInj e = inj[i];
   const int dx = depth(e.x, nbl, nx), dy = depth(e.y, nbl, ny), dz = depth(e.z, nbl, nz);
   const float b = bscale * static_cast<float>(dx * dx + dy * dy + dz * dz);
-  const float s = A[e.off] * e.w * val[e.col] / (1.f + b);
-  atomicAdd(p + e.off, s);
-  atomicAdd(q + e.off, s);
+  const float s = coef[e.off].x * e.w * val[e.col] / (1.f + b);
+  atomicAdd(&u[e.off].x, s);
+  atomicAdd(&u[e.off].y, s);
 }
 
+// Rows [row0, row0 + rows) of the padded grid (row = z Ny + y) between the
+// (p, q) pairs and a dense array of one of the two fields (f = 0: p, 1: q)
+// that starts at row row0.
+__global__ void k_tti_field(float2* __restrict__ u, float* __restrict__ dense, int Nx, int pitch,
+                            size_t row0, int f, int to_user) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= Nx) return;
+  float* cell = reinterpret_cast<float*>(u + (row0 + blockIdx.y) * pitch + x) + f;
+  float* user = dense + static_cast<size_t>(blockIdx.y) * Nx + x;
+  if (to_user)
+    *user = *cell;
+  else
+    *cell = *user;
+}
+
+// Launches one step on the resident CTAs (*ctas, found by the first call).
 template <int R>
-cudaError_t launch_q(const tti::QMaps& M, const tti::QArgs& qa, dim3 grid, cudaStream_t s) {
-  static unsigned long long done = 0;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (!(done & (1ull << (dev & 63)))) {
-    cudaError_t e = cudaFuncSetAttribute(tti::k_tti_q<R>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(tti::QGeom<R>::SMEM));
+cudaError_t launch_q(const tti::QMaps& M, const tti::QArgs& qa, int* ctas, cudaStream_t s) {
+  if (*ctas == 0) {
+    int dev = 0, sms = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (!e) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (!e)
+      e = cudaFuncSetAttribute(tti::k_tti_q<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               int(tti::QGeom<R>::SMEM));
+    if (!e)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tti::k_tti_q<R>, tti::kQT,
+                                                        tti::QGeom<R>::SMEM);
     if (e) return e;
-    done |= 1ull << (dev & 63);
+    // at least 2R planes per share: each run of planes first enters 2R
+    const long long units = (long long)qa.cols * qa.Nz;
+    *ctas = int(std::max<long long>(
+        1, std::min<long long>((long long)std::max(per, 1) * sms, units / (2 * R))));
   }
-  tti::k_tti_q<R><<<grid, tti::kQT, tti::QGeom<R>::SMEM, s>>>(M, qa);
+  tti::k_tti_q<R><<<*ctas, tti::kQT, tti::QGeom<R>::SMEM, s>>>(M, qa);
   return cudaGetLastError();
 }
 
-cudaError_t launch_q_r(int R, const tti::QMaps& M, const tti::QArgs& qa, dim3 grid,
+cudaError_t launch_q_r(int R, const tti::QMaps& M, const tti::QArgs& qa, int* ctas,
                        cudaStream_t s) {
   count_launch();
   switch (R) {
-    case 1: return launch_q<1>(M, qa, grid, s);
-    case 2: return launch_q<2>(M, qa, grid, s);
-    case 3: return launch_q<3>(M, qa, grid, s);
-    case 4: return launch_q<4>(M, qa, grid, s);
-    case 5: return launch_q<5>(M, qa, grid, s);
-    case 6: return launch_q<6>(M, qa, grid, s);
-    case 7: return launch_q<7>(M, qa, grid, s);
-    case 8: return launch_q<8>(M, qa, grid, s);
+    case 1: return launch_q<1>(M, qa, ctas, s);
+    case 2: return launch_q<2>(M, qa, ctas, s);
+    case 3: return launch_q<3>(M, qa, ctas, s);
+    case 4: return launch_q<4>(M, qa, ctas, s);
+    case 5: return launch_q<5>(M, qa, ctas, s);
+    case 6: return launch_q<6>(M, qa, ctas, s);
+    case 7: return launch_q<7>(M, qa, ctas, s);
+    case 8: return launch_q<8>(M, qa, ctas, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -306,17 +335,37 @@ fd_status tables(fd_tti t, const fd_points* src, const fd_points* rec) {
   return FD_OK;
 }
 
-fd_status copy_state(fd_tti t, float* dev, void* user, bool to_user) {
-  cudaMemcpy3DParms p;
-  memset(&p, 0, sizeof(p));
-  cudaPitchedPtr dv = make_cudaPitchedPtr(dev, size_t(t->pitch) * 4, t->Nx * 4, t->Ny);
-  cudaPitchedPtr us = make_cudaPitchedPtr(user, size_t(t->Nx) * 4, t->Nx * 4, t->Ny);
-  p.srcPtr = to_user ? dv : us;
-  p.dstPtr = to_user ? us : dv;
-  p.extent = make_cudaExtent(size_t(t->Nx) * 4, t->Ny, t->Nz);
-  p.kind = cudaMemcpyDefault;
-  cudaError_t e = cudaMemcpy3DAsync(&p, t->stream);
-  if (e) return cuda_fail(e, "wavefield copy");
+// One field of a state (f = 0: p, 1: q) between its pairs and a dense padded
+// array of the caller, device memory directly, host memory through a staging
+// buffer in pieces of whole rows.
+fd_status copy_state(fd_tti t, float2* dev, int f, void* user, bool to_user) {
+  const size_t rows = size_t(t->Ny) * t->Nz;
+  const bool on_device = is_device_ptr(user);
+  const size_t row_bytes = size_t(t->Nx) * 4;
+  const size_t most = 65535;  // rows of one launch
+  const size_t piece =
+      std::min(on_device ? most : std::max<size_t>(1, std::min(most, kStageBytes / row_bytes)),
+               rows);
+  cudaError_t e;
+  if (!on_device && (e = t->stage_in.ensure(piece * row_bytes)))
+    return cuda_fail(e, "state staging");
+  for (size_t r = 0; r < rows; r += piece) {
+    const size_t n = std::min(piece, rows - r);
+    char* u = static_cast<char*>(user) + r * row_bytes;
+    float* dense = static_cast<float*>(on_device ? static_cast<void*>(u) : t->stage_in.p);
+    if (!on_device && !to_user) {
+      e = cudaMemcpyAsync(dense, u, n * row_bytes, cudaMemcpyHostToDevice, t->stream);
+      if (e) return cuda_fail(e, "wavefield copy");
+    }
+    k_tti_field<<<dim3((t->Nx + 127) / 128, unsigned(n)), 128, 0, t->stream>>>(
+        dev, dense, t->Nx, t->pitch, r, f, to_user ? 1 : 0);
+    count_launch();
+    if ((e = cudaGetLastError())) return cuda_fail(e, "wavefield copy");
+    if (!on_device && to_user) {
+      e = cudaMemcpyAsync(u, dense, n * row_bytes, cudaMemcpyDeviceToHost, t->stream);
+      if (e) return cuda_fail(e, "wavefield copy");
+    }
+  }
   return FD_OK;
 }
 
@@ -345,8 +394,6 @@ fd_status propagate(fd_tti t, int n0, int nsteps, const fd_points* src, const fl
       drec = static_cast<float*>(t->stage_rec.p);
     }
   }
-  // the step kernel's arguments; its z chunks are cut so that the launch
-  // fills at least four waves of the resident CTAs
   tti::QArgs qa;
   memset(&qa, 0, sizeof(qa));
   qa.err = static_cast<int*>(t->err.p);
@@ -361,43 +408,29 @@ fd_status propagate(fd_tti t, int n0, int nsteps, const fd_points* src, const fl
   qa.spin_limit = t->spin_limit;
   qa.bscale = t->bscale;
   for (int j = 0; j <= kMaxR; ++j) {
-    qa.c[j] = j <= t->R ? float(t->c[j]) : 0.f;
-    qa.d[j] = j <= t->R ? float(t->d1[j]) : 0.f;
+    qa.c[j].x = qa.c[j].y = j <= t->R ? float(t->c[j]) : 0.f;
+    qa.d[j].x = qa.d[j].y = j <= t->R ? float(t->d1[j]) : 0.f;
   }
-  {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long cols = (long long)((t->Nx + tti::kQX - 1) / tti::kQX) *
-                           ((t->Ny + tti::kQY - 1) / tti::kQY);
-    const long long want = 4LL * (t->R <= 4 ? 2 : 1) * std::max(sms, 1);
-    int chunks = int(std::max<long long>(1, (want + cols - 1) / cols));
-    chunks = std::min(chunks, std::max(1, t->Nz / (8 * t->R)));
-    qa.zchunk = (t->Nz + chunks - 1) / chunks;
-  }
-  const dim3 qgrid((t->Nx + tti::kQX - 1) / tti::kQX, (t->Ny + tti::kQY - 1) / tti::kQY,
-                   (t->Nz + qa.zchunk - 1) / qa.zchunk);
+  qa.cols_y = (t->Ny + tti::kQY - 1) / tti::kQY;
+  qa.cols = qa.cols_y * ((t->Nx + tti::kQX - 1) / tti::kQX);
   if (t->profiling) cudaEventRecord(t->ev0, t->stream);
   for (int s = 0; s < nsteps; ++s) {
     const int cur = t->cur;
     if (nrec) {
       k_tti_gather<<<(nrec + 127) / 128, 128, 0, t->stream>>>(
-          t->p[cur], static_cast<const TtiRec*>(t->rec.p), nrec, drec + size_t(s) * nrec);
+          t->u[cur], static_cast<const TtiRec*>(t->rec.p), nrec, drec + size_t(s) * nrec);
       count_launch();
     }
     tti::QMaps M;
-    M.halo_p = t->halo_p[cur];
-    M.halo_q = t->halo_q[cur];
-    M.prev_p = t->tile_p[cur ^ 1];
-    M.prev_q = t->tile_q[cur ^ 1];
+    M.halo = t->halo[cur];
+    M.prev = t->tile[cur ^ 1];
     M.coef = t->coef_map;
-    qa.pn = t->p[cur ^ 1];
-    qa.qn = t->q[cur ^ 1];
-    if ((e = launch_q_r(t->R, M, qa, qgrid, t->stream))) return cuda_fail(e, "TTI step launch");
+    qa.out = t->u[cur ^ 1];
+    if ((e = launch_q_r(t->R, M, qa, &t->ctas, t->stream))) return cuda_fail(e, "TTI step launch");
     if (t->n_inj) {
       k_tti_inject<<<(t->n_inj + 127) / 128, 128, 0, t->stream>>>(
           static_cast<const TtiInj*>(t->inj.p), t->n_inj, dval + size_t(n0 + s) * nsrc, t->coef,
-          t->bscale, t->d.nbl, t->d.nx, t->d.ny, t->d.nz, t->p[cur ^ 1], t->q[cur ^ 1]);
+          t->bscale, t->d.nbl, t->d.nx, t->d.ny, t->d.nz, t->u[cur ^ 1]);
       count_launch();
     }
     t->cur = cur ^ 1;
@@ -476,12 +509,11 @@ fd_status fd_tti_create(const fd_grid_desc* d, fd_tti* out) {
     t->own_stream = true;
   }
   for (int b = 0; b < 2 && !st; ++b) {
-    e = dev_alloc(reinterpret_cast<void**>(&t->p[b]), t->ncell * 4);
-    if (!e) e = dev_alloc(reinterpret_cast<void**>(&t->q[b]), t->ncell * 4);
+    e = dev_alloc(reinterpret_cast<void**>(&t->u[b]), t->ncell * sizeof(float2));
     if (e) st = cuda_fail(e, "wavefield allocation");
   }
   if (!st) {
-    e = dev_alloc(reinterpret_cast<void**>(&t->coef), 6 * t->ncell * 4);
+    e = dev_alloc(reinterpret_cast<void**>(&t->coef), 3 * t->ncell * sizeof(float2));
     if (!e) e = t->scratch.ensure(64);
     if (!e) e = t->err.ensure(16);
     if (!e) e = cudaMemsetAsync(t->err.p, 0, 16, t->stream);
@@ -489,28 +521,24 @@ fd_status fd_tti_create(const fd_grid_desc* d, fd_tti* out) {
   }
   t->spin_limit = default_spin_limit();
   if (!st) {
-    // tensor maps of the TMA kernel: staged planes with the x halo rounded
-    // up to four floats and R rows, per-point tiles, the six model fields
-    // stacked along z
-    const int W = tti::kQX + 2 * ((t->R + 3) / 4 * 4), H = tti::kQY + 2 * t->R;
+    // tensor maps of the step kernel: staged planes with the x halo rounded
+    // up to two cells and R rows, per-point tiles (rows of pairs are rows of
+    // twice as many floats), the model
+    const int W = tti::kQX + 2 * tti::q_halo_x(t->R);
     for (int b = 0; b < 2 && !st; ++b) {
-      st = make_map(&t->halo_p[b], t->p[b], t->Nx, t->Ny, t->Nz, t->pitch, W, H);
-      if (!st) st = make_map(&t->halo_q[b], t->q[b], t->Nx, t->Ny, t->Nz, t->pitch, W, H);
+      const float* u = reinterpret_cast<const float*>(t->u[b]);
+      st = make_map(&t->halo[b], u, 2 * t->Nx, t->Ny, t->Nz, 2 * t->pitch, 2 * W, tti::kQY + 2 * t->R);
       if (!st)
-        st = make_map(&t->tile_p[b], t->p[b], t->Nx, t->Ny, t->Nz, t->pitch, tti::kQX, tti::kQY);
-      if (!st)
-        st = make_map(&t->tile_q[b], t->q[b], t->Nx, t->Ny, t->Nz, t->pitch, tti::kQX, tti::kQY);
+        st = make_map(&t->tile[b], u, 2 * t->Nx, t->Ny, t->Nz, 2 * t->pitch, 2 * tti::kQX, tti::kQY);
     }
     if (!st)
-      st = make_map(&t->coef_map, t->coef, t->Nx, t->Ny, 6 * t->Nz, t->pitch, tti::kQX,
-                    tti::kQY);
+      st = make_map(&t->coef_map, reinterpret_cast<const float*>(t->coef), 2 * t->Nx, t->Ny,
+                    3 * t->Nz, 2 * t->pitch, 2 * tti::kQX, tti::kQY);
   }
   if (!st) {
-    for (int b = 0; b < 2 && !e; ++b) {
-      e = cudaMemsetAsync(t->p[b], 0, t->ncell * 4, t->stream);
-      if (!e) e = cudaMemsetAsync(t->q[b], 0, t->ncell * 4, t->stream);
-    }
-    if (!e) e = cudaMemsetAsync(t->coef, 0, 6 * t->ncell * 4, t->stream);
+    for (int b = 0; b < 2 && !e; ++b)
+      e = cudaMemsetAsync(t->u[b], 0, t->ncell * sizeof(float2), t->stream);
+    if (!e) e = cudaMemsetAsync(t->coef, 0, 3 * t->ncell * sizeof(float2), t->stream);
     if (!e) e = cudaEventCreate(&t->ev0);
     if (!e) e = cudaEventCreate(&t->ev1);
     if (!e) e = cudaStreamSynchronize(t->stream);
@@ -528,10 +556,8 @@ fd_status fd_tti_destroy(fd_tti t) {
   if (!t) return FD_OK;
   cudaSetDevice(t->d.device);
   if (t->stream) cudaStreamSynchronize(t->stream);
-  for (int b = 0; b < 2; ++b) {
-    if (t->p[b]) cudaFree(t->p[b]);
-    if (t->q[b]) cudaFree(t->q[b]);
-  }
+  for (int b = 0; b < 2; ++b)
+    if (t->u[b]) cudaFree(t->u[b]);
   if (t->coef) cudaFree(t->coef);
   for (DevBuf* b : {&t->inj, &t->rec, &t->stage_val, &t->stage_rec, &t->stage_in, &t->scratch,
                     &t->err})
@@ -600,10 +626,8 @@ fd_status fd_tti_set_model(fd_tti t, const float* vp, const float* epsilon, cons
   } else {
     t->bscale = 0.f;
   }
-  for (int b = 0; b < 2 && !e; ++b) {
-    e = cudaMemsetAsync(t->p[b], 0, t->ncell * 4, t->stream);
-    if (!e) e = cudaMemsetAsync(t->q[b], 0, t->ncell * 4, t->stream);
-  }
+  for (int b = 0; b < 2 && !e; ++b)
+    e = cudaMemsetAsync(t->u[b], 0, t->ncell * sizeof(float2), t->stream);
   if (!e) e = cudaStreamSynchronize(t->stream);
   if (e) return cuda_fail(e, "model set-up");
   t->cur = 0;
@@ -617,8 +641,7 @@ fd_status fd_tti_forward(fd_tti t, const fd_points* src, const float* wavelet,
   if (!t) return fail(FD_ERR_ARG, "null grid");
   cudaSetDevice(t->d.device);
   for (int b = 0; b < 2; ++b) {
-    cudaError_t e = cudaMemsetAsync(t->p[b], 0, t->ncell * 4, t->stream);
-    if (!e) e = cudaMemsetAsync(t->q[b], 0, t->ncell * 4, t->stream);
+    cudaError_t e = cudaMemsetAsync(t->u[b], 0, t->ncell * sizeof(float2), t->stream);
     if (e) return cuda_fail(e, "wavefield reset");
   }
   t->cur = 0;
@@ -639,10 +662,10 @@ fd_status fd_tti_set_state(fd_tti t, const float* p_prev, const float* p, const 
   if (!t) return fail(FD_ERR_ARG, "null grid");
   cudaSetDevice(t->d.device);
   const float* in[4] = {p_prev, p, q_prev, q};
-  float* dst[4] = {t->p[t->cur ^ 1], t->p[t->cur], t->q[t->cur ^ 1], t->q[t->cur]};
-  for (int f = 0; f < 4; ++f) {
-    if (!in[f]) continue;
-    fd_status st = copy_state(t, dst[f], const_cast<float*>(in[f]), false);
+  for (int i = 0; i < 4; ++i) {
+    if (!in[i]) continue;
+    fd_status st = copy_state(t, t->u[(i & 1) ? t->cur : t->cur ^ 1], i >> 1,
+                              const_cast<float*>(in[i]), false);
     if (st) return st;
   }
   cudaError_t e = cudaStreamSynchronize(t->stream);
@@ -655,10 +678,9 @@ fd_status fd_tti_get_state(fd_tti t, float* p_prev, float* p, float* q_prev, flo
   if (!t) return fail(FD_ERR_ARG, "null grid");
   cudaSetDevice(t->d.device);
   float* out[4] = {p_prev, p, q_prev, q};
-  float* src[4] = {t->p[t->cur ^ 1], t->p[t->cur], t->q[t->cur ^ 1], t->q[t->cur]};
-  for (int f = 0; f < 4; ++f) {
-    if (!out[f]) continue;
-    fd_status st = copy_state(t, src[f], out[f], true);
+  for (int i = 0; i < 4; ++i) {
+    if (!out[i]) continue;
+    fd_status st = copy_state(t, t->u[(i & 1) ? t->cur : t->cur ^ 1], i >> 1, out[i], true);
     if (st) return st;
   }
   cudaError_t e = cudaStreamSynchronize(t->stream);

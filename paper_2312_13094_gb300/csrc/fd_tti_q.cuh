@@ -1,70 +1,111 @@
 // TTI step with register queues and TMA staging (included by fd_tti.cu;
-// Sec. IV-B and App. A, Eq. rot).  Space orders up to 8 run two 256-thread
-// CTAs per SM; the wider stencils, whose queues take about 200 registers,
-// one.
+// Sec. IV-B and App. A, Eq. rot).
 //
-// One point per thread on a 32 x 8 tile, a CTA streaming a run of z planes.
+// The two wavefields are stored interleaved, float2 (p, q) per cell, and every
+// stencil operation runs on the pair as one packed f32x2 instruction: both
+// fields take the same weights, so no lane ever needs a neighbour's half.
+// One point per thread, one warp per tile row, a CTA streaming runs of z planes.
 // Every derivative is split by what it needs:
-//  * the in-plane terms D_xx, D_yy and D_xy of a plane need only that plane,
-//    so they are formed once, when the plane enters (p = k + R for output
-//    plane k), and wait R planes in per-thread register queues;
+//  * the in-plane terms of a plane need only that plane, so they are formed
+//    once, when the plane enters (p = k + R for output plane k): D_xx, D_yy,
+//    the first differences dx and dy, and D_xy as the x difference of dy.
+//    dy of the tile and of R columns on each side goes through shared memory
+//    (two buffers); the halo costs 2R columns on 32, where differences of dx
+//    rows would cost 2R rows on the tile's 4.  With the axis (nx, ny) of the
+//    entering plane they are folded at once into what the update needs,
+//    D_xx p + D_yy p and the in-plane part of H_z of both fields, which wait R
+//    planes in register queues (three floats per plane instead of six);
 //  * the z terms D_zz, D_xz and D_yz are sums over planes k-R .. k+R of the
-//    thread's own u and of its first x and y differences dx, dy, which also
-//    enter with their plane and live in register queues of 2R+1 entries.
-// So shared memory holds only the entering plane of p and q with its halo
-// (one 3D TMA tile load per field into a ring of PF+1 slots), the first x
-// differences of that plane on the tile and its R halo rows (for D_xy, two
-// buffers), and the update's eight per-point values of the output plane
-// (six model fields, p^{n-1}, q^{n-1}; TMA tiles, L2 evict-first, PF+1
-// slots).  Loads outside the grid are zero-filled by the TMA unit (the zero
-// ghost).  Every mbarrier wait is bounded; on expiry the CTA records an
-// error, waits (bounded) for its own copies in flight and returns.
+//    thread's own (p, q), dx and dy, which live in register queues of 2R+1
+//    entries.
+// Shared memory holds a ring of four slots, each with one entering plane, its
+// halo and its (nx, ny), and the update's per-point values of the output plane
+// 2R planes behind (the model and the previous p and q; L2 evict-first), all
+// TMA tiles on one mbarrier, and the dy scratch.  The z loop runs four planes
+// per trip, so that a slot's addresses are constants of the code and three of
+// four planes rename the queues instead of shifting them.  Loads outside the
+// grid are zero-filled by the TMA unit (the zero ghost).
+//
+// A launch is persistent.  The tile columns are numbered along y first.  While
+// there are G of them left for the G CTAs, each CTA streams one whole column,
+// in step with its neighbours, whose halos it then finds in L2; the rest is
+// cut into G equal contiguous shares of (column, plane) units.
+//
+// What bounds it (ncu, 336^3 at SO 8): latency; the FMA pipes are 42 % busy, the
+// shared-memory pipe 55-65 %, DRAM 63 % of the copy rate at 1.07 x the 48 B per
+// point.  The scalar kernel with separate fields that this replaced executed 523
+// instructions per point at SO 8 and 902 at SO 16, this one 250 and 390:
+// 100 steps of 336^3 at SO 8 80.7 -> 46.4 ms (81.7 Gpts/s), 60 steps of
+// 243 x 181 x 207 at SO 16 31.6 -> 13.2 ms (41.4 Gpts/s).  Equal shares of all
+// columns instead of whole waves read 1.67 x the bytes (50.5 ms).
+//
+// Every mbarrier wait is bounded.  A thread whose wait runs out records an
+// error and stops waiting (its later waits return at once), the producer stops
+// issuing, and the CTA leaves at the end of the run after a bounded wait for
+// its copies in flight.
 #pragma once
+
+#include <type_traits>
 
 #include "fd_step.cuh"
 
 namespace fd {
 namespace tti {
 
-constexpr int kQX = 32, kQY = 8, kQT = kQX * kQY;  // tile and threads
-constexpr int kQPF = 2;                             // planes in flight ahead
+// Tile and threads: one warp per row of 32 cells, four rows.  Small CTAs keep
+// the per-plane barrier among four warps; eight rows (less halo per tile, half
+// the CTAs) measured 47.7 against 45.9 ms for 100 steps of 336^3 at SO 8, and
+// 14.2 against 13.3 ms for 60 steps of 243 x 181 x 207 at SO 16.
+constexpr int kQX = 32, kQY = 4, kQT = kQX * kQY;
+constexpr int kQS = 4;  // ring slots = planes per loop trip
+
+// Resident CTAs per SM that the launch bounds ask for.  The queues take
+// 6(2R+1) + 3(R+1) registers.  100 steps of 336^3 (ms): SO 4 with 6 / 5 CTAs
+// 33.0 / 34.2; SO 10 with 3 / 2 52.8 / 64.8; SO 12 with 3 / 2 62.6 / 69.8.
+constexpr int q_ctas(int R) { return R <= 2 ? 6 : (R <= 4 ? 4 : (R <= 6 ? 3 : 2)); }
+// x halo of a staged tile: R rounded up to 2 cells (16-byte aligned TMA x coordinate)
+constexpr int q_halo_x(int R) { return (R + 1) / 2 * 2; }
 
 template <int R>
 struct QGeom {
-  // x halo of the staged tile: R rounded up to 4 floats (16-byte aligned TMA x coordinate)
-  static constexpr int RX = ((R + 3) / 4) * 4;
+  static constexpr int RX = q_halo_x(R);
   static constexpr int W = kQX + 2 * RX, H = kQY + 2 * R;
-  static constexpr uint32_t UBYTES = W * H * 4;
-  static constexpr uint32_t UP = (UBYTES + 127) / 128 * 128;  // one field's staged plane
-  static constexpr int SU = kQPF + 1, SA = kQPF + 1;
-  static constexpr int EH = kQY + 2 * R;  // rows of the dx scratch
-  static constexpr int NE = (EH + kQY - 1) / kQY;  // scratch rows per thread
-  static constexpr int CTAS = R <= 4 ? 2 : 1;       // resident CTAs per SM
-  static constexpr uint32_t XP = (kQX * EH * 4 + 127) / 128 * 128;
-  static constexpr uint32_t TBYTES = kQX * kQY * 4;  // one per-point tile
-  static constexpr uint32_t OFF_X = 2 * SU * UP;      // dx scratch: [field][buffer]
-  static constexpr uint32_t OFF_A = OFF_X + 4 * XP;   // per-point tiles: [slot][8]
-  static constexpr uint32_t OFF_BAR = OFF_A + SA * 8 * TBYTES;
-  static constexpr uint32_t SMEM = OFF_BAR + 8 * (SU + SA) + 128;  // + alignment slack
+  // dy of a row's 2R halo cells: HL groups of HP lanes of the row's warp share
+  // the terms of the cells (HT each); a half warp's loads then hit all banks
+  static constexpr int HP = R == 1 ? 2 : (R == 2 ? 4 : (R <= 4 ? 8 : 16));
+  static constexpr int HL = R == 4 ? 4 : (R >= 2 ? 2 : 1);
+  static constexpr int HT = (R + HL - 1) / HL;
+  static_assert(HP * HL <= 32 && HP >= 2 * R, "one warp per row");
+  static constexpr uint32_t UBYTES = W * H * 8;
+  static constexpr uint32_t TBYTES = kQT * 8;  // a tile of pairs
+  // a slot: the plane, its (nx, ny); the output plane's (A, e2), (dl, nz), (nx, ny), previous
+  // (p, q)
+  static constexpr uint32_t OFF_N = (UBYTES + 127) / 128 * 128;
+  static constexpr uint32_t OFF_C = OFF_N + TBYTES;
+  static constexpr uint32_t OFF_P = OFF_C + 3 * TBYTES;
+  static constexpr uint32_t SLOT = OFF_P + TBYTES;
+  static constexpr uint32_t DP = (W * kQY * 8 + 127) / 128 * 128;
+  static constexpr uint32_t OFF_D = kQS * SLOT;  // dy scratch, two buffers
+  static constexpr uint32_t OFF_BAR = OFF_D + 2 * DP;
+  static constexpr uint32_t SMEM = OFF_BAR + 8 * kQS + 128;  // + alignment slack
 };
 
 struct QMaps {
-  CUtensorMap halo_p, halo_q;  // p^n, q^n: 40 x (8 + 2R) boxes
-  CUtensorMap prev_p, prev_q;  // p^{n-1}, q^{n-1}: 32 x 8 boxes
-  CUtensorMap coef;            // the six model fields stacked along z: 32 x 8 boxes
+  CUtensorMap halo;  // (p, q)^n: W x H boxes of cells
+  CUtensorMap prev;  // (p, q)^{n-1}: tiles of cells
+  CUtensorMap coef;  // (A, e2), (dl, nz), (nx, ny) stacked along z: tiles of cells
 };
 
 struct QArgs {
-  float* pn;  // p^{n-1} in, p^{n+1} out (in place)
-  float* qn;
-  int* err;   // set on an expired wait
+  float2* out;  // (p, q)^{n-1} in, (p, q)^{n+1} out (in place)
+  int* err;     // set on an expired wait
   int Nx, Ny, Nz, pitch;
   int nbl, nx, ny, nz;
-  int zchunk;
+  int cols_y, cols;  // tile columns in y, and in all
   long long spin_limit;
   float bscale;
-  float c[kMaxR + 1];
-  float d[kMaxR + 1];
+  float2 c[kMaxR + 1];  // each weight twice, one per half of a pair
+  float2 d[kMaxR + 1];
 };
 
 __device__ __forceinline__ int qdepth(int g, int nbl, int n) {
@@ -74,15 +115,32 @@ __device__ __forceinline__ int qdepth(int g, int nbl, int n) {
   return d > 0 ? d : 0;
 }
 
-template <int N>
-__device__ __forceinline__ void qpush(float (&q)[N], float v) {
+template <int N, class T>
+__device__ __forceinline__ void qpush(T (&q)[N], T v) {
 #pragma unroll
   for (int i = 0; i < N - 1; ++i) q[i] = q[i + 1];
   q[N - 1] = v;
 }
 
+__device__ __forceinline__ float2 lds2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+  return v;
+}
+
+__device__ __forceinline__ void sts2(uint32_t a, float2 v) {
+  asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+
+// a - b, rounded as a subtraction (the product by -1 is exact)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+}
+
 template <int R>
-__global__ void __launch_bounds__(kQT, QGeom<R>::CTAS)
+__global__ void __launch_bounds__(kQT, q_ctas(R))
     k_tti_q(const __grid_constant__ QMaps M, const __grid_constant__ QArgs a) {
   using G = QGeom<R>;
   extern __shared__ unsigned char qsm_raw[];
@@ -91,231 +149,242 @@ __global__ void __launch_bounds__(kQT, QGeom<R>::CTAS)
       qsm_raw + ((128u - (static_cast<uint32_t>(__cvta_generic_to_shared(qsm_raw)) & 127u)) &
                  127u);
   const uint32_t sbase = smem_u32(qsm);
-  const uint32_t bar_u0 = sbase + G::OFF_BAR, bar_a0 = bar_u0 + 8 * G::SU;
+  const uint32_t bar0 = sbase + G::OFF_BAR;
   const int tid = threadIdx.x, tx = tid % kQX, ty = tid / kQX;
-  const int x0 = blockIdx.x * kQX, y0 = blockIdx.y * kQY;
-  const int z0 = blockIdx.z * a.zchunk;
-  const int z1 = min(z0 + a.zchunk, a.Nz);
-  if (z0 >= z1) return;
-  const int nin = z1 - z0 + 2 * R;  // entering planes z0-R .. z1+R-1
-  const int nout = z1 - z0;
-  constexpr int kAux = 32;
-
-  if (tid == 0) {
-    for (int s = 0; s < G::SU; ++s) mbar_init(bar_u0 + 8 * s, 1);
-    for (int s = 0; s < G::SA; ++s) mbar_init(bar_a0 + 8 * s, 1);
-    fence_mbar_init();
+  // own cell in a staged plane, in the dy scratch and in a tile
+  const uint32_t cown = sbase + 8u * ((ty + R) * G::W + tx + G::RX);
+  const uint32_t cd = sbase + G::OFF_D + 8u * (ty * G::W + tx + G::RX);
+  const uint32_t ctile = sbase + 8u * tid;
+  // dy of the row's halo cells: lane tx takes terms j = hj + 1, hj + 1 + HL, ..
+  // of halo cell hc (weight 0 beyond R and for lanes without a cell)
+  const int hc = min(tx % G::HP, 2 * R - 1), hj = min(tx / G::HP, G::HL - 1);
+  const int hcol = hc < R ? hc - R : kQX + hc - R;  // tile column
+  const uint32_t chalo = sbase + 8u * ((ty + R) * G::W + hcol + G::RX);
+  const uint32_t chd = sbase + G::OFF_D + 8u * (ty * G::W + hcol + G::RX);
+  const bool hwrite = tx < 2 * R;  // (its terms' other groups: lanes tx + HP, ..)
+  float hd[G::HT];
+#pragma unroll
+  for (int m = 0; m < G::HT; ++m) {
+    hd[m] = 0.f;
+#pragma unroll
+    for (int j = 1; j <= R; ++j)
+      if (j == hj + 1 + m * G::HL) hd[m] = a.d[j].x;
   }
-  __syncthreads();
+  const uint32_t hstep = 8u * G::W * (hj + 1);  // row offset of the first term
 
-  // producers: thread 0 the staged planes (entering plane i: z = z0-R+i),
-  // thread 32 the per-point tiles (output plane i: z = z0+i)
-  int iu_next = 0, ia_next = 0;
-  auto issue_u = [&](int i) {
-    if (i >= nin) return;
-    iu_next = i + 1;
-    const int s = i % G::SU;
-    const uint32_t bar = bar_u0 + 8 * s;
-    mbar_expect_tx(bar, 2 * G::UBYTES);
-    const int z = z0 - R + i;
-    tma_load_3d(sbase + (2 * s) * G::UP, &M.halo_p, x0 - G::RX, y0 - R, z, bar);
-    tma_load_3d(sbase + (2 * s + 1) * G::UP, &M.halo_q, x0 - G::RX, y0 - R, z, bar);
-  };
-  auto issue_a = [&](int i) {
-    if (i >= nout) return;
-    ia_next = i + 1;
-    const int s = i % G::SA;
-    const uint32_t bar = bar_a0 + 8 * s;
-    mbar_expect_tx(bar, 8 * G::TBYTES);
-    const int z = z0 + i;
-    const uint32_t dst = sbase + G::OFF_A + s * 8 * G::TBYTES;
-#pragma unroll
-    for (int f = 0; f < 6; ++f)
-      tma_load_3d_stream(dst + f * G::TBYTES, &M.coef, x0, y0, z + f * a.Nz, bar);
-    tma_load_3d_stream(dst + 6 * G::TBYTES, &M.prev_p, x0, y0, z, bar);
-    tma_load_3d_stream(dst + 7 * G::TBYTES, &M.prev_q, x0, y0, z, bar);
-  };
-  if (tid == 0)
-    for (int i = 0; i < G::SU; ++i) issue_u(i);
-  if (tid == kAux)
-    for (int i = 0; i < G::SA; ++i) issue_a(i);
-
-  // register queues per field: own u, dx, dy of planes k-R .. k+R (centre at
-  // R) and D_xx, D_yy, D_xy of planes k .. k+R (centre at 0)
-  float qu[2][2 * R + 1], qdx[2][2 * R + 1], qdy[2][2 * R + 1];
-  float qxx[2][R + 1], qyy[2][R + 1], qxy[2][R + 1];
-#pragma unroll
-  for (int f = 0; f < 2; ++f) {
-#pragma unroll
-    for (int i = 0; i < 2 * R + 1; ++i) qu[f][i] = qdx[f][i] = qdy[f][i] = 0.f;
-#pragma unroll
-    for (int i = 0; i < R + 1; ++i) qxx[f][i] = qyy[f][i] = qxy[f][i] = 0.f;
-  }
-
-  const int gx = x0 + tx, gy = y0 + ty;
-  const bool inside = gx < a.Nx && gy < a.Ny;
-  const int dxy = qdepth(gx, a.nbl, a.nx) * qdepth(gx, a.nbl, a.nx) +
-                  qdepth(gy, a.nbl, a.ny) * qdepth(gy, a.nbl, a.ny);
-  // byte offsets: own point in a staged plane; the scratch rows this thread
-  // fills are e = ty + 8m (scratch row e = staged row e, tile row e - R)
-  const uint32_t cown = 4u * ((ty + R) * G::W + tx + G::RX);
-  const uint32_t cx = 4u * ((ty + R) * kQX + tx);
-  const size_t plane = static_cast<size_t>(a.Ny) * a.pitch;
-  size_t off = static_cast<size_t>(z0) * plane + static_cast<size_t>(gy) * a.pitch + gx;
-
+  // this CTA's share of the last, partial wave of columns
+  const int waves = a.cols / gridDim.x, rest = a.cols - waves * gridDim.x;
+  const long long units = static_cast<long long>(rest) * a.Nz;
+  long long pos = units * blockIdx.x / gridDim.x;
+  const long long hi = units * (blockIdx.x + 1) / gridDim.x;
   bool bad = false;
-  int su = 0;
-  uint32_t pu = 0;
-  int sa = 0;
-  uint32_t pa = 0;
+  long long limit = a.spin_limit;
 
-  // one entering plane: its in-plane terms and first differences into the
-  // queues (one barrier: the dx scratch of both fields); returns false when
-  // the CTA must stop
-  auto enter = [&](int i) -> bool {
-    bad |= !mbar_wait(bar_u0 + 8 * su, pu, a.spin_limit);
-    const int buf = i & 1;
-    float dyo[2], xxo[2], yyo[2], uo[2];
+  for (int w = 0; w < waves || pos < hi; ++w) {
+    int col = w * gridDim.x + blockIdx.x, z0 = 0, z1 = a.Nz;
+    if (w >= waves) {
+      col = waves * gridDim.x + static_cast<int>(pos / a.Nz);
+      z0 = static_cast<int>(pos % a.Nz);
+      z1 = static_cast<int>(min(static_cast<long long>(a.Nz), z0 + (hi - pos)));
+      pos += z1 - z0;
+    }
+    const int x0 = col / a.cols_y * kQX, y0 = col % a.cols_y * kQY;
+    const int nout = z1 - z0, nin = nout + 2 * R;  // entering planes z0-R .. z1+R-1
+
+    if (tid == 0) {
+      for (int s = 0; s < kQS; ++s) mbar_init(bar0 + 8 * s, 1);
+      fence_mbar_init();
+    }
+    __syncthreads();
+
+    // producer (thread 0): entering plane i (z = z0-R+i) into slot i mod 4,
+    // with the per-point values of output plane i - 2R
+    int next = 0;
+    auto issue = [&](int i, int s) {
+      if (i >= nin || bad) return;
+      next = i + 1;
+      const uint32_t bar = bar0 + 8 * s, dst = sbase + s * G::SLOT;
+      const int z = z0 - R + i;
+      // the axis of planes that are output planes of this run
+      const bool axis = i >= R && i < R + nout, outp = i >= 2 * R;
+      mbar_expect_tx(bar, G::UBYTES + ((axis ? 1 : 0) + (outp ? 4 : 0)) * G::TBYTES);
+      tma_load_3d(dst, &M.halo, 2 * (x0 - G::RX), y0 - R, z, bar);
+      if (axis) tma_load_3d(dst + G::OFF_N, &M.coef, 2 * x0, y0, z + 2 * a.Nz, bar);
+      if (outp) {
 #pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      const uint32_t P = sbase + (2 * su + f) * G::UP;
-      const float u0 = lds1(P + cown);
-      float xx = a.c[0] * u0, yy = a.c[0] * u0, dy = 0.f;
+        for (int f = 0; f < 3; ++f)
+          tma_load_3d_stream(dst + G::OFF_C + f * G::TBYTES, &M.coef, 2 * x0, y0,
+                             z - R + f * a.Nz, bar);
+        tma_load_3d_stream(dst + G::OFF_P, &M.prev, 2 * x0, y0, z - R, bar);
+      }
+    };
+    if (tid == 0)
+      for (int i = 0; i < kQS; ++i) issue(i, i);
+
+    // register queues: own (p, q), dx, dy of planes k-R .. k+R (centre at R);
+    // the in-plane H_z of both fields and D_xx p + D_yy p of planes k .. k+R
+    // (centre at 0)
+    float2 qu[2 * R + 1], qdx[2 * R + 1], qdy[2 * R + 1], qh[R + 1];
+    float ql[R + 1];
+#pragma unroll
+    for (int i = 0; i < 2 * R + 1; ++i) qu[i] = qdx[i] = qdy[i] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < R + 1; ++i) {
+      qh[i] = make_float2(0.f, 0.f);
+      ql[i] = 0.f;
+    }
+
+    const int gx = x0 + tx, gy = y0 + ty;
+    const bool inside = gx < a.Nx && gy < a.Ny;
+    const int dxv = qdepth(gx, a.nbl, a.nx), dyv = qdepth(gy, a.nbl, a.ny);
+    float2* po = a.out + (static_cast<size_t>(z0) * a.Ny + gy) * a.pitch + gx;
+    const size_t plane = static_cast<size_t>(a.Ny) * a.pitch;
+    // damping of the current output plane: b - 1 and 1 / (1 + b), formed again
+    // only when the plane's depth in the layer changes
+    int dz_of = -1;
+    float bm1 = -1.f, binv = 1.f;
+
+    // plane i, staged in slot s, enters: its first differences and (planes that
+    // will be output planes) in-plane terms go into the queues; one barrier
+    float2 zz, xz, yz;  // z sums of the output plane
+    auto enter = [&](int i, int s, auto inplane, auto zpart) {
+      constexpr bool kIn = decltype(inplane)::value;
+      if (!mbar_wait(bar0 + 8 * s, (i / kQS) & 1, limit)) {
+        bad = true;
+        limit = 0;
+      }
+      // the z sums but for their last term, which enters with this plane:
+      // independent work in the shadow of the loads below (4 % at SO 8 and 16)
+      if (decltype(zpart)::value) {
+        zz = __fmul2_rn(a.c[0], qu[R + 1]);
+        xz = yz = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 1; j < R; ++j) {
+          zz = __ffma2_rn(a.c[j], __fadd2_rn(qu[R + 1 + j], qu[R + 1 - j]), zz);
+          xz = __ffma2_rn(a.d[j], sub2(qdx[R + 1 + j], qdx[R + 1 - j]), xz);
+          yz = __ffma2_rn(a.d[j], sub2(qdy[R + 1 + j], qdy[R + 1 - j]), yz);
+        }
+      }
+      const uint32_t P = cown + s * G::SLOT;
+      const uint32_t D = cd + (s & 1) * G::DP;
+      const float2 u0 = lds2(P);
+      float2 xx = __fmul2_rn(a.c[0], u0), yy = xx;
+      float2 dx = make_float2(0.f, 0.f), dy = dx, hxy = dx, nn = dx;
 #pragma unroll
       for (int j = 1; j <= R; ++j) {
-        const float xp = lds1(P + cown + 4 * j), xm = lds1(P + cown - 4 * j);
-        const float yp = lds1(P + cown + 4 * j * G::W), ym = lds1(P + cown - 4 * j * G::W);
-        xx = fmaf(a.c[j], xp + xm, xx);
-        yy = fmaf(a.c[j], yp + ym, yy);
-        dy = fmaf(a.d[j], yp - ym, dy);
+        const float2 xp = lds2(P + 8 * j), xm = lds2(P - 8 * j);
+        if (kIn) xx = __ffma2_rn(a.c[j], __fadd2_rn(xp, xm), xx);
+        dx = __ffma2_rn(a.d[j], sub2(xp, xm), dx);
       }
-      // first x differences of the scratch rows ty + 8m (staged rows)
-      const uint32_t X = sbase + G::OFF_X + (2 * f + buf) * G::XP;
 #pragma unroll
-      for (int m = 0; m < G::NE; ++m) {
-        const int e = ty + m * kQY;
-        if (m == 0 || e < G::EH) {
-          const uint32_t re = 4u * (e * G::W + tx + G::RX);
-          float ex = 0.f;
+      for (int j = 1; j <= R; ++j) {
+        const float2 yp = lds2(P + 8 * j * G::W), ym = lds2(P - 8 * j * G::W);
+        if (kIn) yy = __ffma2_rn(a.c[j], __fadd2_rn(yp, ym), yy);
+        dy = __ffma2_rn(a.d[j], sub2(yp, ym), dy);
+      }
+      if (kIn) {
+        sts2(D, dy);
+        float2 e = make_float2(0.f, 0.f);
 #pragma unroll
-          for (int j = 1; j <= R; ++j)
-            ex = fmaf(a.d[j], lds1(P + re + 4 * j) - lds1(P + re - 4 * j), ex);
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(X + 4u * (e * kQX + tx)), "f"(ex)
-                       : "memory");
+        for (int m = 0; m < G::HT; ++m) {
+          // terms beyond R (R not a multiple of HL) read the last one again
+          const uint32_t o = (m + 1) * G::HL <= R || hj + 1 + m * G::HL <= R
+                                 ? hstep + 8u * G::W * G::HL * m
+                                 : 8u * G::W * R;
+          const uint32_t h = chalo + s * G::SLOT;
+          e = __ffma2_rn(dup2(hd[m]), sub2(lds2(h + o), lds2(h - o)), e);
+        }
+#pragma unroll
+        for (int o = G::HP; o < G::HP * G::HL; o *= 2)
+          e = __fadd2_rn(e, make_float2(__shfl_xor_sync(0xffffffffu, e.x, o),
+                                        __shfl_xor_sync(0xffffffffu, e.y, o)));
+        if (hwrite) sts2(chd + (s & 1) * G::DP, e);
+        nn = lds2(ctile + s * G::SLOT + G::OFF_N);
+        hxy = __ffma2_rn(dup2(nn.x * nn.x), xx, __fmul2_rn(dup2(nn.y * nn.y), yy));
+      }
+      __syncthreads();
+      if (kIn) {
+        float2 xy = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 1; j <= R; ++j)
+          xy = __ffma2_rn(a.d[j], sub2(lds2(D + 8 * j), lds2(D - 8 * j)), xy);
+        hxy = __ffma2_rn(dup2(2.f * nn.x * nn.y), xy, hxy);
+        qpush(qh, hxy);
+        qpush(ql, xx.x + yy.x);
+      }
+      qpush(qu, u0);
+      qpush(qdx, dx);
+      qpush(qdy, dy);
+    };
+
+    // planes below the first output plane, then those up to its own R-th
+    // neighbour; a slot is refilled one plane later, when the next barrier
+    // shows that every thread is past it
+#pragma unroll 1
+    for (int i = 0; i < R; ++i) {
+      enter(i, i % kQS, std::false_type(), std::false_type());
+      if (tid == 0) issue(i + kQS, i % kQS);
+    }
+#pragma unroll 1
+    for (int i = R; i < 2 * R; ++i) {
+      enter(i, i % kQS, std::true_type(), std::false_type());
+      if (tid == 0) issue(i + kQS, i % kQS);
+    }
+
+    // The slot of output plane k also holds its per-point values, read after
+    // the plane's barrier: it is refilled behind the next plane's barrier.
+    for (int k0 = 0; k0 < nout; k0 += kQS) {
+#pragma unroll
+      for (int t = 0; t < kQS; ++t) {
+        const int k = k0 + t;
+        if (k >= nout) goto done;
+        {
+          constexpr int kFirst = 2 * R % kQS;
+          const int s = (kFirst + t) % kQS;
+          // the last R planes of a run are entered for their z terms only;
+          // their axis is not loaded, and what is formed from it is not used
+          enter(k + 2 * R, s, std::true_type(), std::true_type());
+          if (tid == 0 && k > 0) issue(k + 2 * R - 1 + kQS, (s + kQS - 1) % kQS);
+          const int dz = qdepth(z0 + k, a.nbl, a.nz);
+          if (dz != dz_of) {
+            dz_of = dz;
+            const float b = a.bscale * static_cast<float>(dxv * dxv + dyv * dyv + dz * dz);
+            bm1 = b - 1.f;
+            binv = 1.f / (1.f + b);  // exactly 1 outside the layer
+          }
+          const uint32_t T = ctile + s * G::SLOT;
+          const float2 ae = lds2(T + G::OFF_C);                  // A, e2
+          const float2 dn = lds2(T + G::OFF_C + G::TBYTES);      // dl, nz
+          const float2 nn = lds2(T + G::OFF_C + 2 * G::TBYTES);  // nx, ny
+          const float2 um = lds2(T + G::OFF_P), uc = qu[R];
+          zz = __ffma2_rn(a.c[R], __fadd2_rn(qu[2 * R], qu[0]), zz);
+          xz = __ffma2_rn(a.d[R], sub2(qdx[2 * R], qdx[0]), xz);
+          yz = __ffma2_rn(a.d[R], sub2(qdy[2 * R], qdy[0]), yz);
+          // H_z of both fields, then H_0 p = Laplacian - H_z
+          const float nz = dn.y, nz2 = 2.f * nz, dl = dn.x;
+          float2 hz = __ffma2_rn(dup2(nz * nz), zz, qh[0]);
+          hz = __ffma2_rn(dup2(nz2 * nn.x), xz, hz);
+          hz = __ffma2_rn(dup2(nz2 * nn.y), yz, hz);
+          const float h0 = (ql[0] + zz.x) - hz.x;
+          const float2 r = make_float2(fmaf(ae.y, h0, dl * hz.y), fmaf(dl, h0, hz.y));
+          const float2 un = __ffma2_rn(dup2(ae.x), r,
+                                       __ffma2_rn(dup2(bm1), um, __fadd2_rn(uc, uc)));
+          if (inside) *po = __fmul2_rn(un, dup2(binv));
+          po += plane;
         }
       }
-      uo[f] = u0;
-      xxo[f] = xx;
-      yyo[f] = yy;
-      dyo[f] = dy;
     }
-    if (__syncthreads_or(bad)) return false;
-    // every thread is past this plane's staged tiles and the previous
-    // plane's compute: refill this slot and the last output plane's tiles
-    if (tid == 0) issue_u(i + G::SU);
-    if (tid == kAux && i > 2 * R) issue_a(i - 2 * R - 1 + G::SA);
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      const uint32_t X = sbase + G::OFF_X + (2 * f + buf) * G::XP;
-      float xy = 0.f;
-#pragma unroll
-      for (int j = 1; j <= R; ++j)
-        xy = fmaf(a.d[j], lds1(X + cx + 4 * j * kQX) - lds1(X + cx - 4 * j * kQX), xy);
-      // the own row's first x difference is scratch row ty + R, written before
-      // the barrier (the same sum in the same order)
-      qpush(qu[f], uo[f]);
-      qpush(qdx[f], lds1(X + cx));
-      qpush(qdy[f], dyo[f]);
-      qpush(qxx[f], xxo[f]);
-      qpush(qyy[f], yyo[f]);
-      qpush(qxy[f], xy);
-    }
-    su = (su + 1 == G::SU) ? 0 : su + 1;
-    pu ^= (su == 0) ? 1u : 0u;
-    return true;
-  };
-
-  for (int i = 0; i < 2 * R; ++i)
-    if (!enter(i)) goto fail;
-
-  // four planes per loop trip: the compiler renames the queues for three of
-  // them instead of shifting
-#pragma unroll 4
-  for (int k = 0; k < nout; ++k) {
-    if (!enter(k + 2 * R)) goto fail;
-    bad |= !mbar_wait(bar_a0 + 8 * sa, pa, a.spin_limit);
-    {
-      const uint32_t T = sbase + G::OFF_A + sa * 8 * G::TBYTES + 4u * (ty * kQX + tx);
-      const float A = lds1(T), e2 = lds1(T + G::TBYTES), dl = lds1(T + 2 * G::TBYTES);
-      const float nx = lds1(T + 3 * G::TBYTES), ny = lds1(T + 4 * G::TBYTES),
-                  nz = lds1(T + 5 * G::TBYTES);
-      const float pm = lds1(T + 6 * G::TBYTES), qm = lds1(T + 7 * G::TBYTES);
-      float D[2][6];
-#pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        float zz = a.c[0] * qu[f][R], xz = 0.f, yz = 0.f;
-#pragma unroll
-        for (int j = 1; j <= R; ++j) {
-          zz = fmaf(a.c[j], qu[f][R + j] + qu[f][R - j], zz);
-          xz = fmaf(a.d[j], qdx[f][R + j] - qdx[f][R - j], xz);
-          yz = fmaf(a.d[j], qdy[f][R + j] - qdy[f][R - j], yz);
-        }
-        D[f][0] = qxx[f][0];
-        D[f][1] = qyy[f][0];
-        D[f][2] = zz;
-        D[f][3] = qxy[f][0];
-        D[f][4] = xz;
-        D[f][5] = yz;
-      }
-      const float wxx = nx * nx, wyy = ny * ny, wzz = nz * nz;
-      const float wxy = 2.f * nx * ny, wxz = 2.f * nx * nz, wyz = 2.f * ny * nz;
-      const float* dp = D[0];
-      const float* dq = D[1];
-      const float lap_p = dp[0] + dp[1] + dp[2];
-      const float hz_p = wxx * dp[0] + wyy * dp[1] + wzz * dp[2] + wxy * dp[3] + wxz * dp[4] +
-                         wyz * dp[5];
-      const float hz_q = wxx * dq[0] + wyy * dq[1] + wzz * dq[2] + wxy * dq[3] + wxz * dq[4] +
-                         wyz * dq[5];
-      const float h0_p = lap_p - hz_p;
-      const float rp = e2 * h0_p + dl * hz_q;
-      const float rq = dl * h0_p + hz_q;
-      const int dz = qdepth(z0 + k, a.nbl, a.nz);
-      const float b = a.bscale * static_cast<float>(dxy + dz * dz);
-      const float pc = qu[0][R], qc = qu[1][R];
-      // outside the layer b = 0 and the division by 1 + b is exact: skipped
-      float np_ = 2.f * pc - (1.f - b) * pm + A * rp;
-      float nq_ = 2.f * qc - (1.f - b) * qm + A * rq;
-      if (b != 0.f) {
-        np_ = np_ / (1.f + b);
-        nq_ = nq_ / (1.f + b);
-      }
-      if (inside) {
-        a.pn[off] = np_;
-        a.qn[off] = nq_;
-      }
-    }
-    off += plane;
-    sa = (sa + 1 == G::SA) ? 0 : sa + 1;
-    pa ^= (sa == 0) ? 1u : 0u;
-  }
-  // every issued copy has been waited for (the entering planes up to nin-1,
-  // the per-point tiles up to nout-1); release the barriers
-  __syncthreads();
-  if (tid == 0) {
-    for (int s = 0; s < G::SU; ++s) mbar_inval(bar_u0 + 8 * s);
-    for (int s = 0; s < G::SA; ++s) mbar_inval(bar_a0 + 8 * s);
-  }
-  return;
-
-fail:
-  if (tid == 0) {
-    atomicOr(a.err, 1);
-    for (int i = max(0, iu_next - G::SU); i < iu_next; ++i)
-      mbar_wait(bar_u0 + 8 * (i % G::SU), (i / G::SU) & 1, a.spin_limit);
-  }
-  if (tid == kAux) {
-    for (int i = max(0, ia_next - G::SA); i < ia_next; ++i)
-      mbar_wait(bar_a0 + 8 * (i % G::SA), (i / G::SA) & 1, a.spin_limit);
+  done:
+    // every issued copy has been waited for, but where a wait ran out: there
+    // the producer waits (bounded) for its copies in flight
+    if (bad) atomicOr(a.err, 1);
+    if (tid == 0 && bad)
+      for (int i = max(0, next - kQS); i < next; ++i)
+        mbar_wait(bar0 + 8 * (i % kQS), (i / kQS) & 1, a.spin_limit);
+    // release the barriers for the next run
+    if (__syncthreads_or(bad)) return;
+    if (tid == 0)
+      for (int s = 0; s < kQS; ++s) mbar_inval(bar0 + 8 * s);
   }
 }
 

@@ -145,3 +145,53 @@ def test_errors(fd):
         st = g.forward(np.array([[1e4, 0.0, 0.0]]), w["wavelet"], w["rec"], rec)
         assert st == fd.FD_ERR_ARG
         fd.check(g.forward(w["src"], w["wavelet"], w["rec"], rec), "fd_tti_forward")
+
+
+@pytest.mark.parametrize("so", [6, 10, 14])
+def test_orders_between_the_powers_of_two(fd, so):
+    """Radii whose row halo is not a power of two wide (the lanes that share
+    one halo cell's terms are then not all in use)."""
+    w = wl.tti_workload(n=(35, 27, 24), so=so, nbl=5, nt=30, seed=9)
+    rec, p, q = run_gpu(fd, w)
+    ref = otti.forward(ogrid(w), *model(w), w["nt"], w["src"], w["wavelet"], w["rec"])
+    assert rel(rec, ref["rec"]) <= TOL, rel(rec, ref["rec"])
+    assert rel(p, ref["p"]) <= TOL, rel(p, ref["p"])
+    assert rel(q, ref["q"]) <= TOL, rel(q, ref["q"])
+
+
+def test_more_columns_than_resident_ctas(fd):
+    """Whole waves of columns followed by shares of the rest: 620 tile columns,
+    one step from a random state, element by element."""
+    w = wl.tti_workload(n=(61, 1237, 20), so=8, nbl=1, nt=1)
+    g0 = ogrid(w)
+    st = [wl.random_state(g0.padded_shape, 60 + i).astype(np.float32) for i in range(4)]
+    ref = otti.forward(g0, *model(w), 1, np.zeros((0, 3)), np.zeros((1, 0)), np.zeros((0, 3)),
+                       state=st)
+    with fd.TtiGrid.from_workload(w) as g:
+        g.set_model(*model(w))
+        g.set_state(*st)
+        fd.check(g.propagate(0, 1), "fd_tti_propagate")
+        out = [np.zeros(g0.padded_shape, np.float32) for _ in range(2)]
+        g.get_state(p=out[0], q=out[1])
+    for got, want in ((out[0], ref["p"]), (out[1], ref["q"])):
+        assert np.abs(got - want).max() <= 2e-6 * np.abs(want).max()
+
+
+def test_state_round_trip_in_pieces(fd):
+    """More rows than one conversion launch takes, from host and device arrays."""
+    import torch
+    n = (37, 262, 259)
+    with fd.TtiGrid(n, 10.0, 4, 0, 1.0, 1) as g:
+        shp = g.padded_shape
+        st = [wl.random_state(shp, 80 + i).astype(np.float32) for i in range(4)]
+        g.set_state(*st)
+        dev = [torch.zeros(shp, device="cuda") for _ in range(4)]
+        g.get_state(*dev)
+        torch.cuda.synchronize()
+        for a, b in zip(dev, st):
+            np.testing.assert_array_equal(a.cpu().numpy(), b)
+        g.set_state(p=dev[2], q_prev=dev[1])
+        out = [np.zeros(shp, np.float32) for _ in range(4)]
+        g.get_state(*out)
+    for got, want in zip(out, (st[0], st[2], st[1], st[3])):
+        np.testing.assert_array_equal(got, want)
