@@ -411,6 +411,11 @@ fd_status propagate(fd_tti t, int n0, int nsteps, const fd_points* src, const fl
     qa.c[j].x = qa.c[j].y = j <= t->R ? float(t->c[j]) : 0.f;
     qa.d[j].x = qa.d[j].y = j <= t->R ? float(t->d1[j]) : 0.f;
   }
+  // the centre weight that the FP32 weights c_j need, as hi + lo
+  double c0 = 0.0;
+  for (int j = 1; j <= t->R; ++j) c0 -= 2.0 * qa.c[j].x;
+  qa.c[0].x = qa.c[0].y = float(c0);
+  qa.c0lo.x = qa.c0lo.y = float(c0 - qa.c[0].x);
   qa.cols_y = (t->Ny + tti::kQY - 1) / tti::kQY;
   qa.cols = qa.cols_y * ((t->Nx + tti::kQX - 1) / tti::kQX);
   if (t->profiling) cudaEventRecord(t->ev0, t->stream);

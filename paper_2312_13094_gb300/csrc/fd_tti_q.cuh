@@ -35,8 +35,8 @@
 // shared-memory pipe 55-65 %, DRAM 63 % of the copy rate at 1.07 x the 48 B per
 // point.  The scalar kernel with separate fields that this replaced executed 523
 // instructions per point at SO 8 and 902 at SO 16, this one 250 and 390:
-// 100 steps of 336^3 at SO 8 80.7 -> 46.4 ms (81.7 Gpts/s), 60 steps of
-// 243 x 181 x 207 at SO 16 31.6 -> 13.2 ms (41.4 Gpts/s).  Equal shares of all
+// 100 steps of 336^3 at SO 8 80.7 -> 47.1 ms (80.5 Gpts/s), 60 steps of
+// 243 x 181 x 207 at SO 16 31.6 -> 13.4 ms (40.9 Gpts/s).  Equal shares of all
 // columns instead of whole waves read 1.67 x the bytes (50.5 ms).
 //
 // Every mbarrier wait is bounded.  A thread whose wait runs out records an
@@ -105,6 +105,7 @@ struct QArgs {
   long long spin_limit;
   float bscale;
   float2 c[kMaxR + 1];  // each weight twice, one per half of a pair
+  float2 c0lo;          // the centre weight is c[0] + c0lo
   float2 d[kMaxR + 1];
 };
 
@@ -239,14 +240,18 @@ __global__ void __launch_bounds__(kQT, q_ctas(R))
     const int dxv = qdepth(gx, a.nbl, a.nx), dyv = qdepth(gy, a.nbl, a.ny);
     float2* po = a.out + (static_cast<size_t>(z0) * a.Ny + gy) * a.pitch + gx;
     const size_t plane = static_cast<size_t>(a.Ny) * a.pitch;
-    // damping of the current output plane: b - 1 and 1 / (1 + b), formed again
+    // damping of the current output plane: 1 - b and 1 / (1 + b), formed again
     // only when the plane's depth in the layer changes
     int dz_of = -1;
-    float bm1 = -1.f, binv = 1.f;
+    float omb = 1.f, binv = 1.f;
 
     // plane i, staged in slot s, enters: its first differences and (planes that
     // will be output planes) in-plane terms go into the queues; one barrier
     float2 zz, xz, yz;  // z sums of the output plane
+    // the second derivatives' centre term: -2 sum_j c_j of the FP32 weights, as
+    // two FP32 numbers, so that a constant field has none (one FP32 centre
+    // weight leaves a row sum of ~1e-7, which adds up over the steps)
+    auto centre = [&](float2 u) { return __ffma2_rn(a.c[0], u, __fmul2_rn(a.c0lo, u)); };
     auto enter = [&](int i, int s, auto inplane, auto zpart) {
       constexpr bool kIn = decltype(inplane)::value;
       if (!mbar_wait(bar0 + 8 * s, (i / kQS) & 1, limit)) {
@@ -256,7 +261,7 @@ __global__ void __launch_bounds__(kQT, q_ctas(R))
       // the z sums but for their last term, which enters with this plane:
       // independent work in the shadow of the loads below (4 % at SO 8 and 16)
       if (decltype(zpart)::value) {
-        zz = __fmul2_rn(a.c[0], qu[R + 1]);
+        zz = centre(qu[R + 1]);
         xz = yz = make_float2(0.f, 0.f);
 #pragma unroll
         for (int j = 1; j < R; ++j) {
@@ -268,7 +273,7 @@ __global__ void __launch_bounds__(kQT, q_ctas(R))
       const uint32_t P = cown + s * G::SLOT;
       const uint32_t D = cd + (s & 1) * G::DP;
       const float2 u0 = lds2(P);
-      float2 xx = __fmul2_rn(a.c[0], u0), yy = xx;
+      float2 xx = kIn ? centre(u0) : make_float2(0.f, 0.f), yy = xx;
       float2 dx = make_float2(0.f, 0.f), dy = dx, hxy = dx, nn = dx;
 #pragma unroll
       for (int j = 1; j <= R; ++j) {
@@ -349,7 +354,7 @@ __global__ void __launch_bounds__(kQT, q_ctas(R))
           if (dz != dz_of) {
             dz_of = dz;
             const float b = a.bscale * static_cast<float>(dxv * dxv + dyv * dyv + dz * dz);
-            bm1 = b - 1.f;
+            omb = 1.f - b;
             binv = 1.f / (1.f + b);  // exactly 1 outside the layer
           }
           const uint32_t T = ctile + s * G::SLOT;
@@ -367,9 +372,15 @@ __global__ void __launch_bounds__(kQT, q_ctas(R))
           hz = __ffma2_rn(dup2(nz2 * nn.y), yz, hz);
           const float h0 = (ql[0] + zz.x) - hz.x;
           const float2 r = make_float2(fmaf(ae.y, h0, dl * hz.y), fmaf(dl, h0, hz.y));
-          const float2 un = __ffma2_rn(dup2(ae.x), r,
-                                       __ffma2_rn(dup2(bm1), um, __fadd2_rn(uc, uc)));
-          if (inside) *po = __fmul2_rn(un, dup2(binv));
+          // (1+b) u+ = 2u - (1-b) u- + A r as an increment of u,
+          //   u+ = u + ((1-b) (u - u-) + A r) / (1+b):
+          // u - u- is exact or nearly so, and the rounding of the terms and of
+          // the reciprocal is relative to the increment, not to u.  Rounding
+          // 2u - u- at the size of u was a third to a half of the error against
+          // FP64 (60 steps of 110 x 90 x 100 at SO 16, FP32 emulated term by term:
+          // 4.3e-7 to 5.1e-7 of 5.7e-7 to 1.1e-6; the final rounding the rest).
+          const float2 inc = __ffma2_rn(dup2(ae.x), r, __fmul2_rn(dup2(omb), sub2(uc, um)));
+          if (inside) *po = __ffma2_rn(inc, dup2(binv), uc);
           po += plane;
         }
       }
