@@ -31,236 +31,424 @@ constexpr int OW1 = 0, OB1 = OW1 + H * NIN, OW2 = OB1 + H, OB2 = OW2 + H * H,
               OW3 = OB2 + H, OB3 = OW3 + NOUT * H, NPARAM = OB3 + NOUT;
 static_assert(NPARAM == FD_MLP_NPARAM, "parameter layout");
 constexpr int SAMPLE = FD_MLP_SAMPLE;  // x[4] T[4] y w
-constexpr int CHUNK = 128;            // samples per block iteration = threads
-constexpr int LD = H + 1;             // padded row of the activation tiles
 
 struct TaylorC {
   float c[RL + 1];
 };
 
-__device__ __forceinline__ void load_params(float* sp, const float* __restrict__ p) {
-  for (int i = threadIdx.x; i < NPARAM; i += blockDim.x) sp[i] = p[i];
+// ---------------------------------------------------------------------------
+// One block works on chunks of S = 64 samples with 256 threads as register
+// tiles: thread (sg, ug) = (tid / 16, tid % 16) holds samples 4 sg .. 4 sg + 3
+// by units 4 ug .. 4 ug + 3, and the three 64 x 64 x 64 contractions (z2 = W2 h1,
+// dh1 = W2^T dz2, dW2 = dz2^T h1) run over two float4 shared loads per 16 FMAs.
+// Everything that belongs to a tile's own points (h2, the output layer, dz2, dz1
+// and the gradients of W1, W3 and the biases) stays in registers; the sixteen
+// lanes that share four samples sit in one half warp, so the output layer's
+// sums over units are shuffles.
+//
+// What bounds it: shared-memory reads (two 128-bit loads per 16 FMAs; the FMAs
+// alone, 14 336 per sample forward and backward, would take 23 us of the 61 us
+// below).  One thread per sample, the former layout, read one shared word per
+// FMA and kept four warps per SM; here 16 warps per SM share each operand.
+// Loss and gradient of 65 536 samples: 196 -> 83 us a call, of which the kernel
+// 61 us; per-cell weights of 230 x 213 x 181 cells with the shot that follows:
+// 18.1 -> 15.8 ms.
+//
+// Only s_j = (o_j + o_{j+4}) / 2 enters the coefficients, so o_j + o_{j+4} is
+// one sum and dL/do_j = dL/do_{j+4} is formed once.  (Adding the two weight rows
+// beforehand would round each weight the same way for every sample, which
+// showed in the error of loss and gradient.)
+// ---------------------------------------------------------------------------
+constexpr int S = 64;         // samples per chunk
+constexpr int NTHR = 256;     // threads per block
+constexpr int NSUB = 8;       // samples per warp: the unit in which work is dealt out
+
+// Offsets (floats) of the block's shared memory: parameters, then (gradient
+// only) W2 as stored, the activation tiles and two staged sample chunks.
+constexpr int SM_W1 = 0, SM_B1 = SM_W1 + 4 * H, SM_B2 = SM_B1 + H, SM_W3 = SM_B2 + H,
+              SM_B3 = SM_W3 + NOUT * H, SM_W2T = SM_B3 + NOUT, SM_H1T = SM_W2T + H * H,
+              SM_FWD = SM_H1T + H * S,
+              SM_W2 = SM_FWD, SM_H1 = SM_W2 + H * H, SM_D2 = SM_H1 + S * H,
+              SM_D2T = SM_D2 + S * H, SM_SMP = SM_D2T + H * S,
+              SM_GRAD = SM_SMP + 2 * S * SAMPLE;
+static_assert(SM_W2T % 4 == 0 && SM_SMP % 4 == 0, "float4 tiles");
+
+// Float4 block of the transposed tiles [unit][sample]: the sample blocks of a
+// row are permuted by the row's unit group, so that sixteen unit groups
+// writing the same sample block touch different banks.
+__device__ __forceinline__ int tblk(int row, int sg) { return row * S + 4 * (sg ^ ((row >> 2) & 15)); }
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ float at4(const float4& v, int i) {
+  return i == 0 ? v.x : (i == 1 ? v.y : (i == 2 ? v.z : v.w));
 }
 
-// o = W3 relu(W2 relu(W1 x + b1) + b2) + b3 for one sample; h1 kept.
-__device__ __forceinline__ void net_forward(const float* sp, const float x[NIN], float h1[H],
-                                            float o[NOUT]) {
+// Parameters into shared memory: W1, W3, biases, W2 transposed (W2T[i][k]) and, to keep, W2 as stored.
+__device__ __forceinline__ void load_params(float* sm, const float* __restrict__ p, bool keep) {
+  for (int i = threadIdx.x; i < 4 * H; i += NTHR) {
+    sm[SM_W1 + i] = p[OW1 + i];
+    sm[SM_W3 + i] = p[OW3 + i];
+    sm[SM_W3 + RL * H + i] = p[OW3 + RL * H + i];
+  }
+  for (int i = threadIdx.x; i < H; i += NTHR) {
+    sm[SM_B1 + i] = p[OB1 + i];
+    sm[SM_B2 + i] = p[OB2 + i];
+  }
+  if (threadIdx.x < NOUT) sm[SM_B3 + threadIdx.x] = p[OB3 + threadIdx.x];
+  // W2 by 4 x 4 blocks, transposed in registers (one block per thread)
+  static_assert(NTHR * 16 == H * H && OW2 % 4 == 0, "one block of W2 per thread");
+  const int kb = threadIdx.x & 15, ub = threadIdx.x >> 4;
+  float4 w[4];
 #pragma unroll
-  for (int i = 0; i < H; ++i) {
-    float z = sp[OB1 + i];
-#pragma unroll
-    for (int c = 0; c < NIN; ++c) z = fmaf(sp[OW1 + i * NIN + c], x[c], z);
-    h1[i] = fmaxf(z, 0.0f);
+  for (int r = 0; r < 4; ++r) {
+    w[r] = *reinterpret_cast<const float4*>(p + OW2 + (4 * kb + r) * H + 4 * ub);
+    if (keep) *reinterpret_cast<float4*>(sm + SM_W2 + (4 * kb + r) * H + 4 * ub) = w[r];
   }
 #pragma unroll
-  for (int o_ = 0; o_ < NOUT; ++o_) o[o_] = sp[OB3 + o_];
-  for (int k = 0; k < H; ++k) {
-    float z = sp[OB2 + k];
+  for (int r = 0; r < 4; ++r)
+    st4(sm + SM_W2T + (4 * ub + r) * H + 4 * kb, at4(w[0], r), at4(w[1], r), at4(w[2], r),
+        at4(w[3], r));
+}
+
+// acc[s][u] += a_s b_u
+__device__ __forceinline__ void outer4(float (&acc)[4][4], const float4& a, const float4& b) {
 #pragma unroll
-    for (int i = 0; i < H; ++i) z = fmaf(sp[OW2 + k * H + i], h1[i], z);
-    const float h2 = fmaxf(z, 0.0f);
+  for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int o_ = 0; o_ < NOUT; ++o_) o[o_] = fmaf(sp[OW3 + o_ * H + k], h2, o[o_]);
+    for (int u = 0; u < 4; ++u) acc[s][u] = fmaf(at4(a, s), at4(b, u), acc[s][u]);
+}
+
+// First layer of the thread's tile: h1 = relu(W1 x + b1) for its four samples
+// and units, into the transposed tile.
+__device__ __forceinline__ void layer1(float* sm, int sg, int ug, const float (&x)[4][NIN],
+                                       float (&h1)[4][4]) {
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const float4 w = ld4(sm + SM_W1 + 4 * (4 * ug + u));
+    const float b = sm[SM_B1 + 4 * ug + u];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      float z = b;
+#pragma unroll
+      for (int c = 0; c < NIN; ++c) z = fmaf(at4(w, c), x[s][c], z);
+      h1[s][u] = fmaxf(z, 0.0f);
+    }
+    st4(sm + SM_H1T + tblk(4 * ug + u, sg), h1[0][u], h1[1][u], h1[2][u], h1[3][u]);
   }
 }
 
-__device__ __forceinline__ void coef_from_out(const float o[NOUT], const TaylorC& t,
-                                              float c[RL], float th[RL]) {
+// acc[s][u] += sum_r T[r][sample s] W[r][unit u] over the 64 rows r of a
+// transposed tile T and of W.
+__device__ __forceinline__ void contract(const float* T, const float* W, int sg, int ug,
+                                         float (&acc)[4][4]) {
+#pragma unroll 4
+  for (int r4 = 0; r4 < H / 4; ++r4) {
+    const float* t = T + 4 * r4 * S + 4 * (sg ^ r4);
+    const float* w = W + 4 * r4 * H + 4 * ug;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) outer4(acc, ld4(t + r * S), ld4(w + r * H));
+  }
+}
+
+// Second layer and output of the thread's tile: h2 (kept) and, in lane
+// (sample 4 sg + (ug >> 2), output j = ug & 3), s_j = (o_j + o_{j+4}) / 2.
+__device__ __forceinline__ float layer2_out(const float* sm, int sg, int ug, float (&h2)[4][4]) {
+  const float4 b2 = ld4(sm + SM_B2 + 4 * ug);
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) h2[s][u] = at4(b2, u);
+  contract(sm + SM_H1T, sm + SM_W2T, sg, ug, h2);
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) h2[s][u] = fmaxf(h2[s][u], 0.0f);
+  // sums over units, reduced and scattered over the half warp: lane bits 3 and 2
+  // end with the sample, bits 1 and 0 with the output
+  auto fold = [&](float lo, float hi, int m) {
+    const bool up = (ug & m) != 0;
+    return (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, m);
+  };
+  float v[RL];
 #pragma unroll
   for (int j = 0; j < RL; ++j) {
-    th[j] = tanhf(0.5f * (o[j] + o[j + RL]));
-    c[j] = t.c[j + 1] * (1.0f + 0.5f * th[j]);
-  }
-}
-
-// ---------------------------------------------------------------------------
-// inference on feature rows: coef[n][4]
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_mlp_coef_rows(const float* __restrict__ params,
-                                                      const float* __restrict__ feat, int n,
-                                                      TaylorC t, float* __restrict__ coef) {
-  __shared__ float sp[NPARAM];
-  load_params(sp, params);
-  __syncthreads();
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    float x[NIN], h1[H], o[NOUT], c[RL], th[RL];
+    const float4 w = ld4(sm + SM_W3 + j * H + 4 * ug);
+    const float4 w4 = ld4(sm + SM_W3 + (j + RL) * H + 4 * ug);
+    float z[4];  // this thread's share, per sample
 #pragma unroll
-    for (int q = 0; q < NIN; ++q) x[q] = feat[size_t(s) * NIN + q];
-    net_forward(sp, x, h1, o);
-    coef_from_out(o, t, c, th);
+    for (int s = 0; s < 4; ++s) {
+      z[s] = 0.f;
 #pragma unroll
-    for (int j = 0; j < RL; ++j) coef[size_t(s) * RL + j] = c[j];
-  }
-}
-
-// inference on every padded cell of a grid: x0 = v dt / h = sqrt(A h^2/h^2) =
-// sqrt(A) because A = dt^2 v^2 / h^2; coefficient field j at coef + j*ncell
-__global__ void __launch_bounds__(128) k_mlp_coef_grid(const float* __restrict__ params,
-                                                      const float* __restrict__ A,
-                                                      size_t ncell, int pitch, int Nx,
-                                                      float x1, float x2, float x3,
-                                                      TaylorC t, float* __restrict__ coef) {
-  __shared__ float sp[NPARAM];
-  load_params(sp, params);
-  __syncthreads();
-  for (size_t i = blockIdx.x * size_t(blockDim.x) + threadIdx.x; i < ncell;
-       i += size_t(gridDim.x) * blockDim.x) {
-    float c[RL], th[RL];
-    if (int(i % pitch) >= Nx) {
-#pragma unroll
-      for (int j = 0; j < RL; ++j) c[j] = t.c[j + 1];
-    } else {
-      float x[NIN] = {sqrtf(A[i]), x1, x2, x3}, h1[H], o[NOUT];
-      net_forward(sp, x, h1, o);
-      coef_from_out(o, t, c, th);
+      for (int u = 0; u < 4; ++u) z[s] = fmaf(at4(w4, u), h2[s][u], fmaf(at4(w, u), h2[s][u], z[s]));
     }
+    v[j] = fold(fold(z[0], z[2], 8), fold(z[1], z[3], 8), 4);
+  }
+  const float o = fold(fold(v[0], v[2], 2), fold(v[1], v[3], 2), 1);
+  return 0.5f * (o + (sm[SM_B3 + (ug & 3)] + sm[SM_B3 + RL + (ug & 3)]));
+}
+
+// ---------------------------------------------------------------------------
+// inference: coefficients of feature rows (coef[n][4]), or of every padded cell
+// of a grid, where x0 = v dt / h = sqrt(A) because A = dt^2 v^2 / h^2 and
+// coefficient field j lies at coef + j * n (columns x >= Nx get the Taylor
+// weights).
+// ---------------------------------------------------------------------------
+template <bool GRID>
+__global__ void __launch_bounds__(NTHR, 3)
+    k_mlp_coef(const float* __restrict__ params, const float* __restrict__ in, size_t n, int pitch,
+               int Nx, float x1, float x2, float x3, TaylorC t, float* __restrict__ coef) {
+  extern __shared__ __align__(16) float sm[];
+  const int tid = threadIdx.x, sg = tid >> 4, ug = tid & 15, j = ug & 3;
+  load_params(sm, params, false);
+  __syncthreads();
+  const float tc = t.c[j + 1];
+  const size_t step = size_t(gridDim.x) * S;
+  const int xstep = GRID ? int(step % pitch) : 0;
+  size_t base = size_t(blockIdx.x) * S;
+  int col = GRID ? int((base + 4 * sg + (ug >> 2)) % pitch) : 0;  // of the lane's own cell
+  for (; base < n; base += step) {
+    float x[4][NIN], h1[4][4], h2[4][4];
 #pragma unroll
-    for (int j = 0; j < RL; ++j) coef[j * ncell + i] = c[j];
+    for (int s = 0; s < 4; ++s) {
+      const size_t i = base + 4 * sg + s;
+      if (GRID) {
+        x[s][0] = i < n ? sqrtf(in[i]) : 0.f;
+        x[s][1] = x1;
+        x[s][2] = x2;
+        x[s][3] = x3;
+      } else {
+#pragma unroll
+        for (int c = 0; c < NIN; ++c) x[s][c] = i < n ? in[i * NIN + c] : 0.f;
+      }
+    }
+    __syncwarp();  // a warp's samples are written and read by the warp alone
+    layer1(sm, sg, ug, x, h1);
+    __syncwarp();
+    const float sj = layer2_out(sm, sg, ug, h2);
+    const size_t i = base + 4 * sg + (ug >> 2);
+    if (i < n) {
+      const float c = tc * (1.0f + 0.5f * tanhf(sj));
+      if (GRID)
+        coef[j * n + i] = col < Nx ? c : tc;
+      else
+        coef[i * RL + j] = c;
+    }
+    if (GRID) {
+      col += xstep;
+      if (col >= pitch) col -= pitch;
+    }
   }
 }
 
 // ---------------------------------------------------------------------------
-// training: fused forward, loss and backward over chunks of 128 samples; the
-// weight gradients are contractions over the chunk done from shared memory and
-// accumulated per thread, then added to the global gradient once per block
+// training: fused forward, loss and backward.  Block b of B takes the NSUB-sample
+// units [b U / B, (b + 1) U / B) of the U units in chunks of S; warps whose
+// samples lie beyond the last chunk's end skip it.  The gradient of W2 (64 x 64)
+// is accumulated in the register tile, all others per tile, and a block adds its
+// sums to the global gradient once, as float4 reductions.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(CHUNK, 1)
+__device__ __forceinline__ void red4(float* p, const float4& v) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+__global__ void __launch_bounds__(NTHR, 2)
     k_mlp_grad(const float* __restrict__ params, const float* __restrict__ samples, int n,
                float inv_n, TaylorC t, float* __restrict__ grad, double* __restrict__ loss) {
-  extern __shared__ float sm[];
-  float* sp = sm;                       // NPARAM
-  float* H1 = sp + NPARAM;              // [CHUNK][LD]  h1, later read for dW2
-  float* H2 = H1 + CHUNK * LD;          // [CHUNK][LD]  h2, then dz2
-  float* D1 = H2 + CHUNK * LD;          // [CHUNK][LD]  dz1
-  float* DO = D1 + CHUNK * LD;          // [CHUNK][NOUT]
-  float* XS = DO + CHUNK * NOUT;        // [CHUNK][NIN]
-  const int tid = threadIdx.x;
-  load_params(sp, params);
-
-  // per-thread ownership of gradient entries
-  const int k2 = tid & 63, half = tid >> 6;        // dW2[k2][32 half + q]
-  const int o3 = tid >> 4, kb3 = (tid & 15) * 4;   // dW3[o3][kb3 + q]
-  const int i1 = tid >> 1, cb1 = (tid & 1) * 2;    // dW1[i1][cb1 + q]
-  float a2[32], a3[4], a1[2], ab1 = 0.f, ab2 = 0.f, ab3 = 0.f;
+  extern __shared__ __align__(16) float sm[];
+  const int tid = threadIdx.x, sg = tid >> 4, ug = tid & 15, j = ug & 3;
+  const long long units = (static_cast<long long>(n) + NSUB - 1) / NSUB;
+  const long long lo = units * blockIdx.x / gridDim.x * NSUB;
+  long long hi = units * (blockIdx.x + 1) / gridDim.x * NSUB;
+  if (hi > n) hi = n;
+  constexpr int NST = (S * SAMPLE + NTHR - 1) / NTHR;  // staged floats per thread
+  auto fetch = [&](long long base, float (&r)[NST]) {
 #pragma unroll
-  for (int q = 0; q < 32; ++q) a2[q] = 0.f;
+    for (int q = 0; q < NST; ++q) {
+      const int e = tid + q * NTHR;
+      const bool ok = e < S * SAMPLE && base * SAMPLE + e < hi * SAMPLE;
+      r[q] = ok ? samples[base * SAMPLE + e] : 0.f;
+    }
+  };
+  auto stage = [&](int buf, const float (&r)[NST]) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) a3[q] = 0.f;
-  a1[0] = a1[1] = 0.f;
+    for (int q = 0; q < NST; ++q) {
+      const int e = tid + q * NTHR;
+      if (e < S * SAMPLE) sm[SM_SMP + buf * S * SAMPLE + e] = r[q];
+    }
+  };
+  float nxt[NST];
+  fetch(lo, nxt);
+  load_params(sm, params, true);
+  const float tc = t.c[j + 1];
+  float a1[4][4], a2[4][4], a3[4][4], ab1[4], ab2[4], ab3 = 0.f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    ab1[q] = ab2[q] = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) a1[q][r] = a2[q][r] = a3[q][r] = 0.f;
+  }
   double lsum = 0.0;
+  stage(0, nxt);
   __syncthreads();
 
-  for (int base = blockIdx.x * CHUNK; base < n; base += gridDim.x * CHUNK) {
-    const int s = base + tid;
-    const bool ok = s < n;
-    float x[NIN], T[RL], y = 0.f, w = 0.f;
+  int buf = 0;
+  for (long long base = lo; base < hi; base += S, buf ^= 1) {
+    const int nv = hi - base < S ? static_cast<int>(hi - base) : S;
+    const bool more = base + S < hi;
+    if (more) fetch(base + S, nxt);
+    const float* smp = sm + SM_SMP + buf * S * SAMPLE;
+    const bool live = (tid >> 5) * NSUB < nv;  // uniform in a warp
+    unsigned m1 = 0;                           // h1 > 0, bit 4 s + u
+    if (live) {
+      float x[4][NIN], h1[4][4];
 #pragma unroll
-    for (int q = 0; q < NIN; ++q) x[q] = ok ? samples[size_t(s) * SAMPLE + q] : 0.f;
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-    for (int q = 0; q < RL; ++q) T[q] = ok ? samples[size_t(s) * SAMPLE + NIN + q] : 0.f;
-    if (ok) {
-      y = samples[size_t(s) * SAMPLE + NIN + RL];
-      w = samples[size_t(s) * SAMPLE + NIN + RL + 1];
-    }
-    // forward, keeping h1 and h2 rows in shared memory
-    float h1[H], o[NOUT];
+        for (int c = 0; c < NIN; ++c) x[s][c] = smp[(4 * sg + s) * SAMPLE + c];
+      layer1(sm, sg, ug, x, h1);
 #pragma unroll
-    for (int i = 0; i < H; ++i) {
-      float z = sp[OB1 + i];
+      for (int s = 0; s < 4; ++s) {
+        st4(sm + SM_H1 + (4 * sg + s) * H + 4 * ug, h1[s][0], h1[s][1], h1[s][2], h1[s][3]);
 #pragma unroll
-      for (int c = 0; c < NIN; ++c) z = fmaf(sp[OW1 + i * NIN + c], x[c], z);
-      h1[i] = fmaxf(z, 0.0f);
-      H1[tid * LD + i] = h1[i];
-    }
+        for (int u = 0; u < 4; ++u) m1 |= h1[s][u] > 0.f ? 1u << (4 * s + u) : 0u;
+      }
+      // a warp's samples of the transposed tiles are read by the warp alone
+      __syncwarp();
+      float h2[4][4];
+      const float sj = layer2_out(sm, sg, ug, h2);
+      // loss and dL/do_j (= dL/do_{j+4}) of sample 4 sg + (ug >> 2)
+      const float* own = smp + (4 * sg + (ug >> 2)) * SAMPLE;
+      const float T = own[NIN + j], y = own[NIN + RL], w = own[NIN + RL + 1];
+      const float th = tanhf(sj);
+      float p = tc * (1.0f + 0.5f * th) * T;
+      p += __shfl_xor_sync(0xffffffffu, p, 1);
+      p += __shfl_xor_sync(0xffffffffu, p, 2);
+      const float r = p - y;
+      if (j == 0) lsum += double(w) * double(r) * double(r);
+      const float dp = 2.0f * w * r * inv_n;
+      const float dout = 0.5f * (dp * T * tc * 0.5f * (1.0f - th * th));
+      ab3 += dout;
+      // dz2 and the gradients of W3 and b2
+      float dz[4][4];
 #pragma unroll
-    for (int o_ = 0; o_ < NOUT; ++o_) o[o_] = sp[OB3 + o_];
-    for (int k = 0; k < H; ++k) {
-      float z = sp[OB2 + k];
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int i = 0; i < H; ++i) z = fmaf(sp[OW2 + k * H + i], h1[i], z);
-      const float h2 = fmaxf(z, 0.0f);
-      H2[tid * LD + k] = h2;
+        for (int u = 0; u < 4; ++u) dz[s][u] = 0.f;
 #pragma unroll
-      for (int o_ = 0; o_ < NOUT; ++o_) o[o_] = fmaf(sp[OW3 + o_ * H + k], h2, o[o_]);
-    }
-    // loss and dL/do
-    float c[RL], th[RL];
-    coef_from_out(o, t, c, th);
-    float p = 0.f;
+      for (int jj = 0; jj < RL; ++jj) {
+        const float4 w3 = ld4(sm + SM_W3 + jj * H + 4 * ug);
+        const float4 w34 = ld4(sm + SM_W3 + (jj + RL) * H + 4 * ug);
 #pragma unroll
-    for (int j = 0; j < RL; ++j) p = fmaf(c[j], T[j], p);
-    const float r = p - y;
-    lsum += double(w) * double(r) * double(r);
-    const float dp = 2.0f * w * r * inv_n;
+        for (int s = 0; s < 4; ++s) {
+          const float d = __shfl_sync(0xffffffffu, dout, 4 * s + jj, 16);
 #pragma unroll
-    for (int j = 0; j < RL; ++j) {
-      const float ds = dp * T[j] * t.c[j + 1] * 0.5f * (1.0f - th[j] * th[j]);
-      DO[tid * NOUT + j] = 0.5f * ds;
-      DO[tid * NOUT + j + RL] = 0.5f * ds;
-    }
+          for (int u = 0; u < 4; ++u) {
+            dz[s][u] = fmaf(at4(w34, u), d, fmaf(at4(w3, u), d, dz[s][u]));
+            a3[jj][u] = fmaf(d, h2[s][u], a3[jj][u]);
+          }
+        }
+      }
 #pragma unroll
-    for (int q = 0; q < NIN; ++q) XS[tid * NIN + q] = x[q];
-    __syncthreads();
-
-    // dW3 and db3 over the chunk
-    for (int ss = 0; ss < CHUNK; ++ss) {
-      const float d = DO[ss * NOUT + o3];
+      for (int s = 0; s < 4; ++s) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) a3[q] = fmaf(d, H2[ss * LD + kb3 + q], a3[q]);
-      if (tid < NOUT) ab3 += DO[ss * NOUT + tid];
-    }
-    __syncthreads();
-
-    // own sample: dz2 (into the H2 row), dh1, dz1
-    float dh1[H];
+        for (int u = 0; u < 4; ++u) {
+          dz[s][u] = h2[s][u] > 0.f ? dz[s][u] : 0.f;
+          ab2[u] += dz[s][u];
+        }
+        st4(sm + SM_D2 + (4 * sg + s) * H + 4 * ug, dz[s][0], dz[s][1], dz[s][2], dz[s][3]);
+      }
 #pragma unroll
-    for (int i = 0; i < H; ++i) dh1[i] = 0.f;
-    for (int k = 0; k < H; ++k) {
-      float g = 0.f;
+      for (int u = 0; u < 4; ++u)
+        st4(sm + SM_D2T + tblk(4 * ug + u, sg), dz[0][u], dz[1][u], dz[2][u], dz[3][u]);
+      __syncwarp();
+      // dz1 and the gradients of W1 and b1
+      float d1[4][4];
 #pragma unroll
-      for (int o_ = 0; o_ < NOUT; ++o_) g = fmaf(sp[OW3 + o_ * H + k], DO[tid * NOUT + o_], g);
-      const float dz2 = H2[tid * LD + k] > 0.f ? g : 0.f;
-      H2[tid * LD + k] = dz2;
+      for (int s = 0; s < 4; ++s)
 #pragma unroll
-      for (int i = 0; i < H; ++i) dh1[i] = fmaf(sp[OW2 + k * H + i], dz2, dh1[i]);
-    }
+        for (int u = 0; u < 4; ++u) d1[s][u] = 0.f;
+      contract(sm + SM_D2T, sm + SM_W2, sg, ug, d1);
 #pragma unroll
-    for (int i = 0; i < H; ++i) D1[tid * LD + i] = h1[i] > 0.f ? dh1[i] : 0.f;
-    __syncthreads();
-
-    // dW2, dW1 and the hidden biases over the chunk
-    for (int ss = 0; ss < CHUNK; ++ss) {
-      const float d2 = H2[ss * LD + k2];
+      for (int s = 0; s < 4; ++s) {
+        float xs[NIN];
 #pragma unroll
-      for (int q = 0; q < 32; ++q) a2[q] = fmaf(d2, H1[ss * LD + 32 * half + q], a2[q]);
-      const float d1 = D1[ss * LD + i1];
-      a1[0] = fmaf(d1, XS[ss * NIN + cb1], a1[0]);
-      a1[1] = fmaf(d1, XS[ss * NIN + cb1 + 1], a1[1]);
-      if (tid < H) {
-        ab1 += D1[ss * LD + tid];
-        ab2 += H2[ss * LD + tid];
+        for (int c = 0; c < NIN; ++c) xs[c] = smp[(4 * sg + s) * SAMPLE + c];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float d = (m1 >> (4 * s + u)) & 1u ? d1[s][u] : 0.f;
+          ab1[u] += d;
+#pragma unroll
+          for (int c = 0; c < NIN; ++c) a1[u][c] = fmaf(d, xs[c], a1[u][c]);
+        }
       }
     }
     __syncthreads();
+    // dW2 over the chunk's samples, in units of a warp's samples (those beyond
+    // the end within a unit carry w = 0, so dz2 = 0)
+    {
+      const int nr = (nv + NSUB - 1) / NSUB * NSUB;
+      const float* D = sm + SM_D2 + 4 * sg;
+      const float* Hs = sm + SM_H1 + 4 * ug;
+      for (int s = 0; s < nr; s += NSUB)
+#pragma unroll
+        for (int q = 0; q < NSUB; ++q) outer4(a2, ld4(D + (s + q) * H), ld4(Hs + (s + q) * H));
+    }
+    if (more) stage(buf ^ 1, nxt);
+    __syncthreads();
   }
 
+  // dW2[4 sg + q][4 ug ..]
 #pragma unroll
-  for (int q = 0; q < 32; ++q) atomicAdd(&grad[OW2 + k2 * H + 32 * half + q], a2[q]);
+  for (int q = 0; q < 4; ++q)
+    red4(grad + OW2 + (4 * sg + q) * H + 4 * ug, make_float4(a2[q][0], a2[q][1], a2[q][2], a2[q][3]));
+  // the others: sums over the sixteen sample groups through shared memory
+  // (the activation tiles are free now), as 161 float4 entries [entry][sg]
+  float* R = sm + SM_W2T;
+  constexpr int E1 = 64, EB1 = 128, EB2 = 144, EB3 = 160, NE = 161;
+  static_assert(NE * 64 <= SM_GRAD - SM_W2T, "reduction scratch");
+  auto put = [&](int e, float a, float b, float c, float d) { st4(R + e * 64 + 4 * sg, a, b, c, d); };
 #pragma unroll
-  for (int q = 0; q < 4; ++q) atomicAdd(&grad[OW3 + o3 * H + kb3 + q], a3[q]);
-  atomicAdd(&grad[OW1 + i1 * NIN + cb1], a1[0]);
-  atomicAdd(&grad[OW1 + i1 * NIN + cb1 + 1], a1[1]);
-  if (tid < H) {
-    atomicAdd(&grad[OB1 + tid], ab1);
-    atomicAdd(&grad[OB2 + tid], ab2);
+  for (int q = 0; q < 4; ++q) {
+    put(q * 16 + ug, a3[q][0], a3[q][1], a3[q][2], a3[q][3]);
+    put(E1 + 4 * ug + q, a1[q][0], a1[q][1], a1[q][2], a1[q][3]);
   }
-  if (tid < NOUT) atomicAdd(&grad[OB3 + tid], ab3);
-  // block sum of the loss
+  put(EB1 + ug, ab1[0], ab1[1], ab1[2], ab1[3]);
+  put(EB2 + ug, ab2[0], ab2[1], ab2[2], ab2[3]);
+  ab3 += __shfl_xor_sync(0xffffffffu, ab3, 4);
+  ab3 += __shfl_xor_sync(0xffffffffu, ab3, 8);
+  if (ug < 4) R[EB3 * 64 + 4 * sg + ug] = ab3;
+  __syncthreads();
+  if (tid < NE) {
+    float4 v = ld4(R + tid * 64);
+    for (int q = 1; q < 16; ++q) {
+      const float4 o = ld4(R + tid * 64 + 4 * q);
+      v.x += o.x;
+      v.y += o.y;
+      v.z += o.z;
+      v.w += o.w;
+    }
+    if (tid < E1) {  // rows j and j + 4 of W3 share their gradient
+      red4(grad + OW3 + 4 * tid, v);
+      red4(grad + OW3 + RL * H + 4 * tid, v);
+    } else if (tid < EB1) {
+      red4(grad + OW1 + 4 * (tid - E1), v);
+    } else if (tid < EB2) {
+      red4(grad + OB1 + 4 * (tid - EB1), v);
+    } else if (tid < EB3) {
+      red4(grad + OB2 + 4 * (tid - EB2), v);
+    } else {
+      red4(grad + OB3, v);
+      red4(grad + OB3 + RL, v);
+    }
+  }
   for (int off = 16; off > 0; off >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, off);
-  if ((tid & 31) == 0) atomicAdd(loss, lsum * double(inv_n));
+  if ((tid & 31) == 0 && lsum != 0.0) atomicAdd(loss, lsum * double(inv_n));
 }
-
-constexpr size_t GRAD_SMEM = sizeof(float) * (NPARAM + 3 * CHUNK * LD + CHUNK * NOUT + CHUNK * NIN);
 
 // Adam (Kingma & Ba, ICLR 2015) with bias correction; step t >= 1.
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
@@ -360,6 +548,10 @@ int sm_count() {
 
 }  // namespace
 
+// gradient and, behind it, the loss: one reset and one read for both
+constexpr size_t GRAD_BYTES = NPARAM * 4 + sizeof(double);
+static_assert(NPARAM * 4 % sizeof(double) == 0, "loss alignment");
+
 struct fd_mlp_s {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -367,8 +559,9 @@ struct fd_mlp_s {
   float* g = nullptr;   // gradient
   float* m = nullptr;   // Adam first moment
   float* v = nullptr;   // Adam second moment
-  double* loss = nullptr;
-  int t = 0;            // Adam step count
+  double* loss = nullptr;  // behind the gradient in its allocation
+  float* host = nullptr;    // pinned image of gradient and loss
+  int t = 0;               // Adam step count
   DevBuf stage, stage2;
 };
 
@@ -378,9 +571,10 @@ fd_status mlp_grid_coefficients(fd_mlp net, const float* A, size_t ncell, int pi
                                 double h, double dt, double f_hz, float* coef,
                                 cudaStream_t s) {
   const TaylorC t = taylor_c();
-  const int grid = std::max(1, std::min<int>(sm_count() * 8, int((ncell + 127) / 128)));
-  k_mlp_coef_grid<<<grid, 128, 0, s>>>(net->p, A, ncell, pitch, Nx, float(h / 10.0),
-                                       float(dt / 1.0), float(f_hz / 10.0), t, coef);
+  const int grid =
+      int(std::max<size_t>(1, std::min<size_t>(size_t(sm_count()) * 3, (ncell + S - 1) / S)));
+  k_mlp_coef<true><<<grid, NTHR, SM_FWD * sizeof(float), s>>>(
+      net->p, A, ncell, pitch, Nx, float(h / 10.0), float(dt / 1.0), float(f_hz / 10.0), t, coef);
   count_launch();
   cudaError_t e = cudaGetLastError();
   if (e) return cuda_fail(e, "learned coefficient inference");
@@ -402,9 +596,11 @@ fd_status fd_mlp_create(int32_t device, const float* params, fd_mlp* out) {
   fd_status st = FD_OK;
   e = cudaStreamCreateWithFlags(&net->stream, cudaStreamDefault);  // see fd_create_grid
   float** bufs[4] = {&net->p, &net->g, &net->m, &net->v};
-  for (int i = 0; i < 4 && !e; ++i) e = dev_alloc(reinterpret_cast<void**>(bufs[i]), NPARAM * 4);
-  if (!e) e = dev_alloc(reinterpret_cast<void**>(&net->loss), 16);
+  for (int i = 0; i < 4 && !e; ++i)
+    e = dev_alloc(reinterpret_cast<void**>(bufs[i]), GRAD_BYTES);
+  if (!e) e = cudaMallocHost(reinterpret_cast<void**>(&net->host), GRAD_BYTES);
   if (!e) {
+    net->loss = reinterpret_cast<double*>(net->g + NPARAM);
     for (int i = 0; i < 4 && !e; ++i) e = cudaMemsetAsync(*bufs[i], 0, NPARAM * 4, net->stream);
     if (!e && params) e = cudaMemcpyAsync(net->p, params, NPARAM * 4, cudaMemcpyDefault,
                                           net->stream);
@@ -425,7 +621,7 @@ fd_status fd_mlp_destroy(fd_mlp net) {
   if (net->stream) cudaStreamSynchronize(net->stream);
   for (float* p : {net->p, net->g, net->m, net->v})
     if (p) cudaFree(p);
-  if (net->loss) cudaFree(net->loss);
+  if (net->host) cudaFreeHost(net->host);
   net->stage.release();
   net->stage2.release();
   if (net->stream) cudaStreamDestroy(net->stream);
@@ -456,30 +652,38 @@ fd_status fd_mlp_set_params(fd_mlp net, const float* in) {
   return FD_OK;
 }
 
-static fd_status mlp_grad_device(fd_mlp net, int64_t n, const float* dsamples, double* loss) {
-  cudaError_t e = cudaMemsetAsync(net->g, 0, NPARAM * 4, net->stream);
-  if (!e) e = cudaMemsetAsync(net->loss, 0, sizeof(double), net->stream);
+static fd_status mlp_grad_device(fd_mlp net, int64_t n, const float* dsamples) {
+  cudaError_t e = cudaMemsetAsync(net->g, 0, GRAD_BYTES, net->stream);
   if (e) return cuda_fail(e, "gradient reset");
   if (n > 0) {
     static bool attr = false;
     if (!attr) {
       e = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               int(GRAD_SMEM));
+                               int(SM_GRAD * sizeof(float)));
       if (e) return cuda_fail(e, "kernel attribute");
       attr = true;
     }
-    const int blocks = int(std::min<int64_t>(sm_count(), (n + CHUNK - 1) / CHUNK));
-    k_mlp_grad<<<blocks, CHUNK, GRAD_SMEM, net->stream>>>(net->p, dsamples, int(n),
-                                                          float(1.0 / double(n)), taylor_c(),
-                                                          net->g, net->loss);
+    // two blocks per SM; a small batch is spread one warp's samples per block
+    const int blocks = int(std::min<int64_t>(2 * sm_count(), (n + NSUB - 1) / NSUB));
+    k_mlp_grad<<<blocks, NTHR, SM_GRAD * sizeof(float), net->stream>>>(
+        net->p, dsamples, int(n), float(1.0 / double(n)), taylor_c(), net->g, net->loss);
     count_launch();
     if ((e = cudaGetLastError())) return cuda_fail(e, "training kernel");
   }
-  if (loss) {
-    e = cudaMemcpyAsync(loss, net->loss, sizeof(double), cudaMemcpyDeviceToHost, net->stream);
-    if (!e) e = cudaStreamSynchronize(net->stream);
-    if (e) return cuda_fail(e, "loss read");
-  }
+  return FD_OK;
+}
+
+// Loss and (grad not null) gradient of the last mlp_grad_device to the caller.
+static fd_status mlp_grad_read(fd_mlp net, double* loss, float* grad) {
+  cudaError_t e = cudaSuccess;
+  const bool dev = grad && is_device_ptr(grad);
+  if (dev) e = cudaMemcpyAsync(grad, net->g, NPARAM * 4, cudaMemcpyDeviceToDevice, net->stream);
+  if (!e && (loss || (grad && !dev)))
+    e = cudaMemcpyAsync(net->host, net->g, GRAD_BYTES, cudaMemcpyDeviceToHost, net->stream);
+  if (!e) e = cudaStreamSynchronize(net->stream);
+  if (e) return cuda_fail(e, "gradient read");
+  if (loss) memcpy(loss, net->host + NPARAM, sizeof(double));
+  if (grad && !dev) memcpy(grad, net->host, NPARAM * 4);
   return FD_OK;
 }
 
@@ -497,14 +701,9 @@ fd_status fd_mlp_loss_grad(fd_mlp net, int64_t n, const float* samples, double* 
     if (e) return cuda_fail(e, "sample upload");
     d = static_cast<const float*>(net->stage.p);
   }
-  fd_status st = mlp_grad_device(net, n, d, loss);
-  if (st) return st;
-  if (grad_out) {
-    cudaError_t e = cudaMemcpyAsync(grad_out, net->g, NPARAM * 4, cudaMemcpyDefault, net->stream);
-    if (!e) e = cudaStreamSynchronize(net->stream);
-    if (e) return cuda_fail(e, "gradient read");
-  }
-  return FD_OK;
+  fd_status st = mlp_grad_device(net, n, d);
+  if (st || (!loss && !grad_out)) return st;
+  return mlp_grad_read(net, loss, grad_out);
 }
 
 static fd_status adam_device(fd_mlp net, float lr) {
@@ -548,7 +747,7 @@ fd_status fd_mlp_train(fd_mlp net, int64_t n, const float* samples, int32_t epoc
   for (int ep = 0; ep < epochs; ++ep) {
     for (int64_t b0 = 0; b0 < n; b0 += batch) {
       const int64_t nb = std::min<int64_t>(batch, n - b0);
-      if ((st = mlp_grad_device(net, nb, d + size_t(b0) * SAMPLE, nullptr))) return st;
+      if ((st = mlp_grad_device(net, nb, d + size_t(b0) * SAMPLE))) return st;
       if ((st = adam_device(net, lr))) return st;
     }
   }
@@ -558,7 +757,8 @@ fd_status fd_mlp_train(fd_mlp net, int64_t n, const float* samples, int32_t epoc
     for (int64_t b0 = 0; b0 < n; b0 += (int64_t(1) << 24)) {
       const int64_t nb = std::min<int64_t>(int64_t(1) << 24, n - b0);
       double l = 0.0;
-      if ((st = mlp_grad_device(net, nb, d + size_t(b0) * SAMPLE, &l))) return st;
+      if ((st = mlp_grad_device(net, nb, d + size_t(b0) * SAMPLE))) return st;
+      if ((st = mlp_grad_read(net, &l, nullptr))) return st;
       total += l * double(nb);
     }
     *loss_out = total / double(n);
@@ -588,8 +788,9 @@ fd_status fd_mlp_coefficients(fd_mlp net, int64_t n, const float* features, floa
     cout = static_cast<float*>(net->stage2.p);
   }
   if (e) return cuda_fail(e, "staging");
-  const int grid = int(std::min<int64_t>(sm_count() * 8, (n + 127) / 128));
-  k_mlp_coef_rows<<<grid, 128, 0, net->stream>>>(net->p, fin, int(n), taylor_c(), cout);
+  const int grid = int(std::min<int64_t>(sm_count() * 3, (n + S - 1) / S));
+  k_mlp_coef<false><<<grid, NTHR, SM_FWD * sizeof(float), net->stream>>>(
+      net->p, fin, size_t(n), 1, 1, 0.f, 0.f, 0.f, taylor_c(), cout);
   count_launch();
   if ((e = cudaGetLastError())) return cuda_fail(e, "inference");
   if (host_out)

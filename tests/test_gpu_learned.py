@@ -66,6 +66,32 @@ def test_loss_gradient_matches_reference(learned, n):
     net.close()
 
 
+@pytest.mark.parametrize("n", [7, 8, 9, 63, 64, 65, 19457])
+def test_loss_gradient_at_the_edges_of_a_block(learned, n):
+    """Sample counts around a warp's eight samples and a chunk's 64, and one
+    that gives every block two chunks, the second partly filled."""
+    th = mlp.init_params(8, scale_out=0.8).astype(np.float32)
+    net = learned.Network(th)
+    S = samples(n, n + 1)
+    loss, g = net.loss_grad(S)
+    rl, rg = mlp.loss_grad(th.astype(np.float64), S.astype(np.float64),
+                           oracle.fd_coefficients(4))
+    assert abs(loss - rl) <= 1e-5 * abs(rl)
+    assert np.linalg.norm(g - rg) <= 1e-4 * np.linalg.norm(rg)
+    net.close()
+
+
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 29185])
+def test_inference_at_the_edges_of_a_chunk(learned, n):
+    th = mlp.init_params(5, scale_out=0.8).astype(np.float32)
+    net = learned.Network(th)
+    X = mlp.features(np.linspace(1.5, 4.5, n), 20.0, 1.6, 12.0).astype(np.float32)
+    got = net.coefficients(X)
+    ref = mlp.coefficients(th.astype(np.float64), X.astype(np.float64), oracle.fd_coefficients(4))
+    assert np.abs(got - ref).max() <= 1e-5 * np.abs(ref).max()
+    net.close()
+
+
 def test_adam_step_matches_reference(fd, learned):
     th = mlp.init_params(7, scale_out=0.8).astype(np.float32)
     net = learned.Network(th)
