@@ -266,6 +266,79 @@ __device__ __forceinline__ void lap4_packed(const float* xr, YN yn, ZN zn, const
   lap[3] = lp[1].y;
 }
 
+// Differences d_j = S_j - 6 u, j = 1..R, of four consecutive x points for the
+// per-point weight modes (arguments as lap4_packed): lap = sum_j c_j d_j, which
+// needs no centre weight.
+template <int R, int XO, class YN, class ZN>
+__device__ __forceinline__ void diffs4(const float* xr, YN yn, ZN zn, float2 (&dj)[R][2]) {
+  const float2 m6 = make_float2(-6.0f, -6.0f);
+#pragma unroll
+  for (int jj = 1; jj <= R; ++jj) {
+    float4 ym, yp;
+    yn(jj, ym, yp);
+    const float4 zm = zn(-jj), zp = zn(jj);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int xa = XO + 2 * p - jj, xb = XO + 2 * p + jj;
+      const float2 sx =
+          (jj & 1) ? make_float2(__fadd_rn(xr[xa], xr[xb]), __fadd_rn(xr[xa + 1], xr[xb + 1]))
+                   : __fadd2_rn(make_float2(xr[xa], xr[xa + 1]), make_float2(xr[xb], xr[xb + 1]));
+      const float2 sy = __fadd2_rn(half2of(ym, p), half2of(yp, p));
+      const float2 sz = __fadd2_rn(half2of(zm, p), half2of(zp, p));
+      const float2 u2 = make_float2(xr[XO + 2 * p], xr[XO + 2 * p + 1]);
+      dj[jj - 1][p] = __ffma2_rn(m6, u2, __fadd2_rn(__fadd2_rn(sx, sy), sz));
+    }
+  }
+}
+
+// sum_j c_j d_j with every point's own weights, cv(j) the four points' c_j.
+template <int R, class CV>
+__device__ __forceinline__ void weigh_cells(const float2 (&dj)[R][2], CV cv, float (&lap)[4]) {
+  float2 lp[2];
+#pragma unroll
+  for (int jj = 1; jj <= R; ++jj) {
+    const float4 c = cv(jj);
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+      lp[p] = (jj == 1) ? __fmul2_rn(half2of(c, p), dj[0][p])
+                        : __ffma2_rn(half2of(c, p), dj[jj - 1][p], lp[p]);
+  }
+  lap[0] = lp[0].x;
+  lap[1] = lp[0].y;
+  lap[2] = lp[1].x;
+  lap[3] = lp[1].y;
+}
+
+// The same with weights interpolated linearly in the table at each point's A
+// (node i at A = lo + i / inv: weights tab[2 i], step to the next tab[2 i + 1]).
+// Point by point, once the differences are there, so that a point's weights
+// live only while they are applied.  The node comes from adding 1.5 * 2^23 to
+// x - 1/2, whose low bits then hold floor(x) (at a node either of its two
+// intervals: the interpolation is continuous); conversion instructions run at
+// an eighth of the rate.
+template <int R>
+__device__ __forceinline__ void weigh_table(const float2 (&dj)[R][2], const float4& A,
+                                            const float4* tab, float lo, float inv, int nodes,
+                                            float (&lap)[4]) {
+  const float top = static_cast<float>(nodes - 1);
+  constexpr float kMagic = 12582912.0f;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const float x = fminf(fmaxf((lane(A, l) - lo) * inv, 0.0f), top);
+    const float m = fminf(fmaxf(x - 0.5f, 0.0f), top - 1.0f) + kMagic;
+    const int i = __float_as_int(m) - __float_as_int(kMagic);
+    const float f = x - (m - kMagic);
+    const float4 t0 = tab[2 * i];
+    const float4 dt = tab[2 * i + 1];
+#pragma unroll
+    for (int jj = 1; jj <= R; ++jj) {
+      const float d = (l & 1) ? dj[jj - 1][l >> 1].y : dj[jj - 1][l >> 1].x;
+      const float c = fmaf(f, lane(dt, jj - 1), lane(t0, jj - 1));
+      lap[l] = (jj == 1) ? c * d : fmaf(c, d, lap[l]);
+    }
+  }
+}
+
 // Leapfrog update of four points where b = 0: u^{n+1} = A(lap + s) + (2u - u^{n-1})
 // with e = A(lap + s), as packed pairs (the roundings of the scalar form).
 __device__ __forceinline__ void update4_inner(const float lap[4], const float src[4],
@@ -603,70 +676,21 @@ __device__ __forceinline__ void run_column(const CUtensorMap* tm_halo,
           // per-point weights c_1..c_R: from the staged coefficient tiles, or
           // interpolated linearly in the table at the point's own
           // A = (v dt / h)^2
-          float ct[4][R];
-          if (MODE == kModeTable) {
-            const float4 At = lds4(abuf + sa * C::TPITCH + ctile);
-            const float top = static_cast<float>(a.tab_nodes - 1);
-#pragma unroll
-            for (int l = 0; l < 4; ++l) {
-              const float x = fminf(fmaxf((lane(At, l) - a.tab_lo) * a.tab_inv, 0.0f), top);
-              const int i = min(static_cast<int>(x), a.tab_nodes - 2);
-              const float f = x - static_cast<float>(i);
-              const float4 t0 = s_tab[2 * i];
-              const float4 dt = s_tab[2 * i + 1];
-#pragma unroll
-              for (int jj = 1; jj <= R; ++jj)
-                ct[l][jj - 1] = fmaf(f, lane(dt, jj - 1), lane(t0, jj - 1));
-            }
-          }
-          if (MODE == kModeTable) {
-            // lane by lane (the sixteen interpolated weights stay live: as
-            // packed pairs they would spill)
-#pragma unroll
-            for (int jj = 1; jj <= R; ++jj) {
-              const float4 ym = lds4(P - 4 * jj * C::W);
-              const float4 yp = lds4(P + 4 * jj * C::W);
-#pragma unroll
-              for (int l = 0; l < 4; ++l) {
-                const float sx = xr[C::RX + l - jj] + xr[C::RX + l + jj];
-                const float sy = lane(ym, l) + lane(yp, l);
-                const float sz = lane(zq(-jj), l) + lane(zq(jj), l);
-                const float d = fmaf(-6.0f, xr[C::RX + l], (sx + sy) + sz);
-                lap[l] = (jj == 1) ? ct[l][jj - 1] * d : fmaf(ct[l][jj - 1], d, lap[l]);
-              }
-            }
+          float2 dj[R][2];
+          diffs4<R, C::RX>(
+              xr,
+              [&](int jj, float4& ym, float4& yp) {
+                ym = lds4(P - 4 * jj * C::W);
+                yp = lds4(P + 4 * jj * C::W);
+              },
+              zq, dj);
+          if (MODE == kModePerCell) {
+            weigh_cells<R>(
+                dj, [&](int jj) { return lds4(cbuf + (sa * NC + jj - 1) * C::TPITCH + ctile); },
+                lap);
           } else {
-          // per-cell weights: lanes (0,1) and (2,3) as packed pairs, each with
-          // its own weights (the roundings of the scalar form, lane by lane)
-          const float2 m6 = make_float2(-6.0f, -6.0f);
-          float2 lp[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-          for (int jj = 1; jj <= R; ++jj) {
-            float4 cv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (MODE == kModePerCell)
-              cv = lds4(cbuf + (sa * NC + (jj - 1)) * C::TPITCH + ctile);
-            const float4 ym = lds4(P - 4 * jj * C::W);
-            const float4 yp = lds4(P + 4 * jj * C::W);
-            const float4 zm = zq(-jj), zp = zq(jj);
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {
-              const int xa = C::RX + 2 * p - jj, xb = C::RX + 2 * p + jj;
-              const float2 sx =
-                  (jj & 1) ? make_float2(__fadd_rn(xr[xa], xr[xb]), __fadd_rn(xr[xa + 1], xr[xb + 1]))
-                           : __fadd2_rn(make_float2(xr[xa], xr[xa + 1]),
-                                        make_float2(xr[xb], xr[xb + 1]));
-              const float2 sy = __fadd2_rn(half2of(ym, p), half2of(yp, p));
-              const float2 sz = __fadd2_rn(half2of(zm, p), half2of(zp, p));
-              const float2 u2 = make_float2(xr[C::RX + 2 * p], xr[C::RX + 2 * p + 1]);
-              const float2 d = __ffma2_rn(m6, u2, __fadd2_rn(__fadd2_rn(sx, sy), sz));
-              const float2 cj = half2of(cv, p);
-              lp[p] = (jj == 1) ? __fmul2_rn(cj, d) : __ffma2_rn(cj, d, lp[p]);
-            }
-          }
-          lap[0] = lp[0].x;
-          lap[1] = lp[0].y;
-          lap[2] = lp[1].x;
-          lap[3] = lp[1].y;
+            weigh_table<R>(dj, lds4(abuf + sa * C::TPITCH + ctile), s_tab, a.tab_lo, a.tab_inv,
+                           a.tab_nodes, lap);
           }
         } else {
           lap4_packed<R, C::RX>(
