@@ -274,8 +274,13 @@ fd_status fd_set_tile(fd_grid grid, int32_t tile_x, int32_t tile_y, int32_t ctas
  *                    depth, so neighbours share halos in L2 however many
  *                    columns there are; the chunk height minimises the load
  *                    of the busiest CTA (a host-side simulation);
- *   FD_SCHED_AUTO    the default: equal shares, except that a grid left on
- *                    its default tile (no fd_set_tile call) is tuned by its
+ *   FD_SCHED_AUTO    the default.  A grid left on its default tile (no
+ *                    fd_set_tile call) of a few million padded cells runs on
+ *                    bricks: one CTA per 32 x 8 x 8 points, staged at once
+ *                    (fd_grid_info then shows the 32 x 8 tile and
+ *                    FD_SCHED_SHARES).  A larger one runs column waves on the
+ *                    32 x 16 or 64 x 8 tile, whichever the simulation finds
+ *                    less loaded, until it is tuned by its
  *                    first fd_forward, fd_adjoint_gradient or fd_backward of
  *                    at least 400 steps: every compiled tile is timed under
  *                    both schedules for a few source-free steps on the
@@ -284,7 +289,7 @@ fd_status fd_set_tile(fd_grid grid, int32_t tile_x, int32_t tile_y, int32_t ctas
  *                    that padded size and kernel mode on that device
  *                    (fd_forward, fd_propagate and the adjoint; the pick is
  *                    cached per process; fd_grid_info shows the tile and
- *                    schedule in use).
+ *                    schedule in use).  After fd_set_tile: equal shares.
  *   FD_SCHED_TEMPORAL  temporal blocking (the paper's Discussion, Sec. IV,
  *                    names it as future work): space orders 4 and 8 with
  *                    uniform weights advance two steps per pass over the
@@ -296,11 +301,10 @@ fd_status fd_set_tile(fd_grid grid, int32_t tile_x, int32_t tile_y, int32_t ctas
  *                    odd step count ends with one single step.  Other space
  *                    orders, per-cell or table weights and decomposed grids
  *                    run single steps with equal shares instead.
- * The adjoint's steps (fd_adjoint, fd_gradient) and table-weight forward
- * steps follow the same choice as plain forward runs (the tuner's tile and
- * schedule once the grid has been tuned); per-cell weight fields always use
- * equal shares on the default tile, and so does an explicit CTA count
- * (fd_set_tile ctas > 0).  Every schedule and tile gives the same results
+ * The adjoint's steps (fd_adjoint, fd_gradient) and the forward steps with
+ * weight tables or per-cell weights follow the same choice as plain forward
+ * runs (per-cell weights are not tuned); an explicit CTA count
+ * (fd_set_tile ctas > 0) always uses equal shares.  Every schedule and tile gives the same results
  * bit for bit.
  * Errors: FD_ERR_ARG (unknown mode). */
 enum { FD_SCHED_AUTO = 0, FD_SCHED_SHARES = 1, FD_SCHED_WAVES = 2, FD_SCHED_TEMPORAL = 3 };

@@ -75,6 +75,7 @@ fd_status adjoint_impl(fd_grid g, const fd_points* src, const float* wavelet,
   // that is a forward run or this one (source-free steps on zeroed
   // wavefields), before the point tables are built for the tile in use
   if (g->auto_tile && !g->tuned && g->sched_mode == FD_SCHED_AUTO && !g->dmp && !g->cart &&
+      !brick_grid(g) &&
       nt >= kTuneMinSteps && g->debug_skip_plane < 0) {
     for (int b = 0; b < 2; ++b)
       if ((e = cudaMemsetAsync(g->F.u[b], 0, cell_bytes, g->stream)))

@@ -177,11 +177,20 @@ struct TileShape {
   int ctas;         // persistent CTAs per sweep (0: resident CTAs per SM x SMs)
 };
 
-// Per-radius launchers, specialised in fd_step_r<R>.cu.
+// Per-radius launchers, specialised in fd_step_r<R>.cu.  pdl: the launch ahead
+// on the stream is a step too, and this one may start before it has finished
+// (it waits for its results itself).
 template <int R>
 cudaError_t launch_sweep_r(const TileShape& t, int mode, const ShotDesc* shots,
                            const long long* prefix, int nshots, const StepOverride& ov,
-                           int grid, cudaStream_t s);
+                           int grid, bool pdl, cudaStream_t s);
+// Brick kernel of small grids (fd_brick.cuh): its tile, the planes of a brick,
+// and one step of a grid on that tile.
+constexpr int kBrickPlanes = 8;
+constexpr TileShape kBrickTile = {8, 8, 1, 0};
+template <int R>
+cudaError_t launch_brick_r(int mode, const ShotDesc* shot, const StepOverride& ov, int Nx, int Ny,
+                           int Nz, bool pdl, cudaStream_t s);
 template <int R>
 int sweep_blocks_per_sm_r(const TileShape& t, int mode);
 

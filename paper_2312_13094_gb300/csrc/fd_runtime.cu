@@ -172,17 +172,17 @@ fd_status build_maps(fd_grid g) {
 // --------------------------------------------------------------------------
 cudaError_t launch_sweep(int R, const TileShape& t, int mode, const ShotDesc* shots,
                          const long long* prefix, int nshots, const StepOverride& ov, int grid,
-                         cudaStream_t s) {
+                         cudaStream_t s, bool pdl) {
   count_launch();
   switch (R) {
-    case 1: return launch_sweep_r<1>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 2: return launch_sweep_r<2>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 3: return launch_sweep_r<3>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 4: return launch_sweep_r<4>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 5: return launch_sweep_r<5>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 6: return launch_sweep_r<6>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 7: return launch_sweep_r<7>(t, mode, shots, prefix, nshots, ov, grid, s);
-    case 8: return launch_sweep_r<8>(t, mode, shots, prefix, nshots, ov, grid, s);
+    case 1: return launch_sweep_r<1>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 2: return launch_sweep_r<2>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 3: return launch_sweep_r<3>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 4: return launch_sweep_r<4>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 5: return launch_sweep_r<5>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 6: return launch_sweep_r<6>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 7: return launch_sweep_r<7>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
+    case 8: return launch_sweep_r<8>(t, mode, shots, prefix, nshots, ov, grid, pdl, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -578,15 +578,42 @@ void fill_desc(fd_grid g, const RunSpec& rs, ShotDesc* d) {
   d->args.out = nullptr;
 }
 
+// Tile of the plain runs of a grid left on its default tile that the tuner has
+// not seen (runs below kTuneMinSteps): it runs under the wave schedule, whose
+// chunk height balances the resident CTAs for any size.  Of the two tiles of
+// 512 points, 32 x 16 and 64 x 8, the one whose busiest CTA has less to do; on a
+// tie 64 x 8 up to SO 4 (its longer rows) and 32 x 16 (its smaller halo) beyond.
+// Measured (us a step, 32 x 16 / 64 x 8 / the equal shares on default_shape
+// that such runs had before): 251 x 197 x 163 SO 8 31.3 / 32.0 / 36.4;
+// 200 x 240 x 280 SO 8 47.7 / 54.8 / 49.8; 190^3 SO 12 36.9 / 37.2 / 57.6;
+// 300^3 SO 4 95.0 / 86.6 / -; 440 x 340 x 370 SO 16 304 / 249 / -.  The predicted
+// loads of the last are 282 and 205 planes.
+static TileShape wave_tile(fd_grid g) {
+  if (g->wave_shape.tx == 0) {
+    const TileShape shapes[2] = {{8, 16, 1, 0}, {16, 8, 2, 0}};
+    long long load[2];
+    for (int i = 0; i < 2; ++i) {
+      const int bx = 4 * shapes[i].tx, by = shapes[i].ty;
+      const int tiles = ((g->Nx + bx - 1) / bx) * ((g->Ny + by - 1) / by);
+      load[i] = wave_load({{0, tiles, g->Nz}}, sweep_ctas(g->R, shapes[i], kModeForward), g->R);
+    }
+    g->wave_shape = shapes[load[1] < load[0] || (load[1] == load[0] && g->R <= 2) ? 1 : 0];
+  }
+  return g->wave_shape;
+}
+
 // FD_SCHED_WAVES runs every forward sweep of the grid on the wave schedule of
-// fd_sched.cu; FD_SCHED_AUTO does so for plain forward runs when the tuner
-// picked it, else the equal-share sweep (lockstep when the columns fit).
+// fd_sched.cu; FD_SCHED_AUTO does so for plain runs on wave_tile and, once the
+// grid is tuned, when the tuner picked it, else the equal-share sweep (lockstep
+// when the columns fit).
 int grid_schedule(fd_grid g, int mode, StepOverride* ov, fd_status* st) {
   *st = FD_OK;
-  const bool tuned_waves = g->sched_mode == FD_SCHED_AUTO && g->tuned && g->tuned_waves &&
-                           g->shape.tx == g->tuned_shape.tx && g->shape.ty == g->tuned_shape.ty;
-  if (mode == kModePerCell || g->shape.ctas > 0 ||
-      !(g->sched_mode == FD_SCHED_WAVES || tuned_waves))
+  bool auto_waves = false;
+  if (g->sched_mode == FD_SCHED_AUTO && (g->tuned ? g->tuned_waves : g->auto_tile)) {
+    const TileShape on = g->tuned ? g->tuned_shape : wave_tile(g);
+    auto_waves = g->shape.tx == on.tx && g->shape.ty == on.ty;
+  }
+  if (g->shape.ctas > 0 || !(g->sched_mode == FD_SCHED_WAVES || auto_waves))
     return 0;
   const int slots = sweep_ctas(g->R, g->shape, mode);
   const long long key[5] = {g->shape.tx, g->shape.ty, g->Nz,
@@ -618,10 +645,44 @@ int grid_schedule(fd_grid g, int mode, StepOverride* ov, fd_status* st) {
   return g->sched_ctas;
 }
 
+// The brick kernel runs grids of up to four million padded cells (five at SO 6,
+// six up to SO 4) that are left to AUTO.  Measured, us a step, bricks / column
+// waves on wave_tile: SO 2 at 5.2, 8.1 M cells 15.5 / 18.0, 24.0 / 23.1; SO 4
+// 18.7 / 19.6, 27.4 / 24.9; SO 6 at 4.1, 5.2 M 16.9 / 18.0, 22.9 / 23.1; SO 8
+// 20.0 / 22.0, 28.3 / 24.0; SO 16 44 / 48, 68 / 52; at 0.3 M cells SO 4
+// 5.3 / 10.8, SO 8 5.2 / 16.1, SO 16 8.9 / 37; weight table at 3.6 M cells
+// 29.7 / 34.5.  Per-cell weights, whose bricks admit two CTAs per SM, up to 2.5 M:
+// 1.0 M cells 15.6 / 29.4, 3.6 M 37.3 / 30.5.
+bool brick_grid(fd_grid g) {
+  const long long most =
+      g->percell ? 2500000 : (g->R <= 2 ? 6000000 : (g->R == 3 ? 5000000 : 4000000));
+  return g->auto_tile && g->sched_mode == FD_SCHED_AUTO && !g->dmp &&
+         !g->cart &&
+         (long long)g->Nx * g->Ny * g->Nz <= most;
+}
+
+static cudaError_t launch_brick(int R, int mode, const ShotDesc* shot, const StepOverride& ov,
+                                int Nx, int Ny, int Nz, bool pdl, cudaStream_t s) {
+  count_launch();
+  switch (R) {
+    case 1: return launch_brick_r<1>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 2: return launch_brick_r<2>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 3: return launch_brick_r<3>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 4: return launch_brick_r<4>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 5: return launch_brick_r<5>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 6: return launch_brick_r<6>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 7: return launch_brick_r<7>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+    case 8: return launch_brick_r<8>(mode, shot, ov, Nx, Ny, Nz, pdl, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
 fd_status use_shape(fd_grid g, bool plain_forward) {
-  const TileShape want = (plain_forward && g->tuned && g->sched_mode == FD_SCHED_AUTO)
-                             ? g->tuned_shape
-                             : g->base_shape;
+  const TileShape want =
+      plain_forward && brick_grid(g) ? kBrickTile
+      : !plain_forward || g->sched_mode != FD_SCHED_AUTO
+          ? g->base_shape
+          : (g->tuned ? g->tuned_shape : (g->auto_tile ? wave_tile(g) : g->base_shape));
   if (want.tx == 0) return FD_OK;  // a grid without a base tile keeps its own
   if (want.tx == g->shape.tx && want.ty == g->shape.ty && want.ctas == g->shape.ctas)
     return FD_OK;
@@ -713,6 +774,15 @@ fd_status autotune_grid(fd_grid g) {
   return use_shape(g, true);
 }
 
+// Sweeps of up to 16 million padded cells may start before the one ahead has
+// finished: 251 x 197 x 163 SO 8 31.3 -> 30.5 us a step, 240^3 SO 16 73.3 -> 72.8.
+// Longer ones lose more than a launch's latency, as CTAs that start where an
+// earlier one ends break up the waves of neighbouring columns: 592^3 SO 8
+// 575 -> 598 us, 380^3 SO 16 251 -> 256 us.
+static bool short_step(fd_grid g) {
+  return (long long)g->Nx * g->Ny * g->Nz <= 16000000;
+}
+
 fd_status run_steps(fd_grid g, const RunSpec& rs) {
   if (rs.nsteps <= 0) return FD_OK;
   cudaError_t e;
@@ -723,10 +793,14 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
   // fall on chunk boundaries), so every CTA walks z in step with its
   // neighbours, which share halos in L2; otherwise equal contiguous shares
   // of all the (tile, plane) units over every resident slot
-  int G = lockstep_ctas(g->R, g->shape, mode, (long long)g->tiles_x * g->tiles_y, g->Nz);
+  const bool brick = brick_grid(g);
+  int G = brick ? 0
+                : lockstep_ctas(g->R, g->shape, mode, (long long)g->tiles_x * g->tiles_y, g->Nz);
   StepOverride sched_ov;
   memset(&sched_ov, 0, sizeof(sched_ov));
-  {
+  if (brick) {
+    if (mode == kModeForward || mode == kModeTable) g->last_sched = FD_SCHED_SHARES;
+  } else {
     fd_status st = FD_OK;
     const int Gs = grid_schedule(g, mode, &sched_ov, &st);
     if (st) return st;
@@ -802,7 +876,10 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
       if (mode == kModeStoreE) ov.e_out = rs.e_base + size_t(t) * g->ncell;
       if (mode == kModeAdjoint)
         ov.e_in = rs.e_base + size_t(rs.e_idx0 + rs.e_idx_step * t) * g->ncell;
-      e = launch_sweep(g->R, g->shape, mode, dshot, dprefix, 1, ov, G, g->stream);
+      // every launch but the first follows a step on the stream
+      e = brick ? launch_brick(g->R, mode, dshot, ov, g->Nx, g->Ny, g->Nz, t > 0, g->stream)
+                : launch_sweep(g->R, g->shape, mode, dshot, dprefix, 1, ov, G, g->stream,
+                               t > 0 && short_step(g));
       if (e) {
         if (use_graph) {
           cudaGraph_t dummy = nullptr;
@@ -1073,9 +1150,9 @@ static fd_status propagate_impl(fd_grid g, int32_t n0, int32_t nsteps, const fd_
   const int nsrc = src ? src->n : 0, nrec = rec ? rec->n : 0;
   if ((nsrc && (!src->xyz || !wavelet)) || (nrec && (!rec->xyz || !rec_out)))
     return fail(FD_ERR_ARG, "points given without their data array");
-  // plain and table-weight forward runs take the tuner's pick (tile and
-  // schedule) for the grid's size; per-cell weight fields keep the base tile
-  fd_status st = use_shape(g, !g->dmp && !g->cart && forward_mode(g) != kModePerCell);
+  // forward runs take the tuner's pick (tile and schedule) for the grid's size
+  // (per-cell weight fields are not tuned: wave_tile)
+  fd_status st = use_shape(g, !g->dmp && !g->cart);
   if (st) return st;
   if (g->dmp) return decomp_propagate(g, n0, nsteps, src, wavelet, rec, rec_out);
   if (g->cart) return cart_propagate(g, n0, nsteps, src, wavelet, rec, rec_out);
@@ -1151,7 +1228,7 @@ fd_status fd_forward(fd_grid g, const fd_points* src, const float* wavelet,
   // are tuned once (on the grid's own kernel), on the zeroed wavefields,
   // which are cleared again afterwards
   if (g->auto_tile && !g->tuned && g->sched_mode == FD_SCHED_AUTO && !g->dmp && !g->cart &&
-      forward_mode(g) != kModePerCell && g->d.nt >= kTuneMinSteps && g->debug_skip_plane < 0) {
+      !brick_grid(g) && forward_mode(g) != kModePerCell && g->d.nt >= kTuneMinSteps && g->debug_skip_plane < 0) {
     fd_status st = autotune_grid(g);
     if (st) return st;
     for (int b = 0; b < 2; ++b) {

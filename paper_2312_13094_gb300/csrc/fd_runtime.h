@@ -59,7 +59,7 @@ struct GraphKey {
   float* e_base;
   int e_idx0, e_idx_step;
   TileShape shape;
-  int ctas;
+  int ctas;  // 0: brick kernel
   void* desc;
   const void* sched;  // work items of a wave-scheduled sweep (nullptr: equal shares)
   int skip;
@@ -132,6 +132,7 @@ struct fd_grid_s {
   bool auto_tile = false;          // no fd_set_tile: plain forward runs may be tuned
   bool tuned = false;              // tuned_shape / tuned_waves hold the tuner's pick
   fd::TileShape tuned_shape = {};
+  fd::TileShape wave_shape = {};   // tile of runs on AUTO that are not tuned (0: not picked yet)
   bool tuned_waves = false;
 };
 
@@ -160,7 +161,10 @@ fd_status autotune_grid(fd_grid g);
 TileShape default_shape(int R, int Nx, int Ny, int Nz);
 cudaError_t launch_sweep(int R, const TileShape& t, int mode, const ShotDesc* shots,
                          const long long* prefix, int nshots, const StepOverride& ov, int grid,
-                         cudaStream_t s);
+                         cudaStream_t s, bool pdl = false);
+// Whether the grid's plain steps (forward, e-storing and adjoint) run on the
+// brick kernel of small grids.
+bool brick_grid(fd_grid g);
 int sweep_ctas(int R, const TileShape& t, int mode);
 // CTAs of one step launch: k z chunks per column when the columns fit in the
 // resident slots (lockstep), else every resident slot; k = slots / columns,

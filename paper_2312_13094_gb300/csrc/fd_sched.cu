@@ -33,53 +33,82 @@ namespace {
 // Chunks of a column of nz planes at target height H: ceil(nz / H).
 int chunks_of(int nz, double H) { return std::max(1, int(std::ceil(nz / H - 1e-9))); }
 
-long long max_load(const std::vector<SchedGrid>& grids, double H, int G, int R, long long* items) {
+// Load of the busiest CTA at target height H, counting 2R + 4 per item.  The
+// tiles of one chunk are consecutive items of one height: whole waves of them
+// add to every CTA alike, the parts of waves at their ends to ranges of CTAs.
+long long max_load(const std::vector<SchedGrid>& grids, double H, int G, int R) {
   const long long over = 2LL * R + 4;
-  std::vector<long long> load(G, 0);
-  long long i = 0;
+  std::vector<long long> step(G + 1, 0);  // differences of the loads along the CTAs
+  long long i = 0, all = 0;
   for (const SchedGrid& g : grids) {
     const int k = chunks_of(g.nz, H);
     for (int j = 0; j < k; ++j) {
-      const long long h = (long long)g.nz * (j + 1) / k - (long long)g.nz * j / k;
-      for (int t = 0; t < g.tiles; ++t, ++i) {
+      const long long v =
+          (long long)g.nz * (j + 1) / k - (long long)g.nz * j / k + over;
+      for (long long left = g.tiles; left > 0;) {
         const long long w = i / G, p = i % G;
-        load[(w & 1) ? G - 1 - p : p] += h + over;
+        long long c = std::min(left, G - p);
+        if (p == 0 && left >= G) {
+          all += v * (left / G);
+          c = left / G * G;
+        } else {
+          const long long lo = (w & 1) ? G - p - c : p;
+          step[lo] += v;
+          step[lo + c] -= v;
+        }
+        i += c;
+        left -= c;
       }
     }
   }
-  *items = i;
-  return *std::max_element(load.begin(), load.end());
+  long long most = 0, sum = 0;
+  for (int c = 0; c < G; ++c) most = std::max(most, sum += step[c]);
+  return all + most;
 }
 
-}  // namespace
-
-int wave_schedule(const std::vector<SchedGrid>& grids, int G, int R,
-                  std::vector<int32_t>& start, std::vector<WorkItem>& items) {
-  start.clear();
-  items.clear();
+// The chunk height with the least loaded busiest CTA, and that load.
+double best_height(const std::vector<SchedGrid>& grids, int G, int R, long long* load) {
   long long planes = 0;
   int nzmax = 1;
   for (const SchedGrid& g : grids) {
     planes += (long long)g.tiles * g.nz;
     nzmax = std::max(nzmax, g.nz);
   }
-  if (G < 1 || planes == 0) return 0;
   // candidate heights: the tallest column in k = 1 .. 64 chunks, and all
   // planes spread over W = 1 .. 64 full waves; none below 4R planes
   std::vector<double> cand;
   for (int k = 1; k <= 64; ++k) cand.push_back(double(nzmax) / k);
   for (int W = 1; W <= 64; ++W) cand.push_back(double(planes) / (double(W) * G));
   double bestH = nzmax;
-  long long n_items = 0;
-  long long best = max_load(grids, bestH, G, R, &n_items);
+  long long best = max_load(grids, bestH, G, R);
   for (double H : cand) {
     if (H > nzmax || H < 4.0 * R) continue;
-    const long long l = max_load(grids, H, G, R, &n_items);
+    const long long l = max_load(grids, H, G, R);
     if (l < best) {
       best = l;
       bestH = H;
     }
   }
+  *load = best;
+  return bestH;
+}
+
+}  // namespace
+
+long long wave_load(const std::vector<SchedGrid>& grids, int G, int R) {
+  long long load = 0;
+  if (G > 0) best_height(grids, G, R, &load);
+  return load;
+}
+
+int wave_schedule(const std::vector<SchedGrid>& grids, int G, int R,
+                  std::vector<int32_t>& start, std::vector<WorkItem>& items) {
+  start.clear();
+  items.clear();
+  long long planes = 0, load = 0;
+  for (const SchedGrid& g : grids) planes += (long long)g.tiles * g.nz;
+  if (G < 1 || planes == 0) return 0;
+  const double bestH = best_height(grids, G, R, &load);
   // the items in wave order, then grouped per CTA
   std::vector<std::vector<WorkItem>> per(G);
   long long i = 0;

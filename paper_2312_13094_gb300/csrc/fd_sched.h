@@ -19,4 +19,8 @@ struct SchedGrid {
 int wave_schedule(const std::vector<SchedGrid>& grids, int G, int R,
                   std::vector<int32_t>& start, std::vector<WorkItem>& items);
 
+// Load of the busiest of the G CTAs of that schedule (planes, and 2R + 4 per
+// item).
+long long wave_load(const std::vector<SchedGrid>& grids, int G, int R);
+
 }  // namespace fd

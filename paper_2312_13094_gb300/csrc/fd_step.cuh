@@ -201,6 +201,17 @@ __device__ __forceinline__ void st_stream(float* p, float a, float b, float c, f
                : "memory");
 }
 
+// Programmatic dependent launch (launches of consecutive steps on one stream):
+// the next step's CTAs may start where this one leaves room, and load what no
+// step writes; pdl_wait returns once the launch before this one has finished
+// and its writes are visible.  Both do nothing in an ordinary launch.
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 __device__ __forceinline__ int sponge_depth(int g, int nbl, int n) {
   int d = nbl - g;
   int e = g - (n + nbl - 1);
@@ -856,6 +867,8 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
   const long long lo = total * blockIdx.x / gridDim.x;
   const long long hi = total * (blockIdx.x + 1) / gridDim.x;
   const int cur = ov.cur;
+  pdl_trigger();
+  pdl_wait();
   int s = 0;
   for (long long pos = lo; pos < hi;) {
     while (pos >= prefix[s + 1]) ++s;
@@ -896,6 +909,8 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
   __shared__ StepArgs sa;
   const int cur = ov.cur;
   const int i1 = ov.item_start[blockIdx.x + 1];
+  pdl_trigger();
+  pdl_wait();
   for (int i = ov.item_start[blockIdx.x]; i < i1; ++i) {
     const WorkItem w = ov.items[i];
     const ShotDesc* S = shots + w.shot;
@@ -913,6 +928,24 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
                                     w.zb + ov.zfirst, w.ze + ov.zfirst, smem);
     __syncthreads();
   }
+}
+
+// Launch that may start before the launch ahead of it on the stream has
+// finished (pdl; the kernel waits for it with pdl_wait).
+template <class... P, class... A>
+cudaError_t launch_step(void (*k)(P...), dim3 grid, int threads, uint32_t smem, bool pdl,
+                        cudaStream_t s, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, args...);
 }
 
 }  // namespace fd

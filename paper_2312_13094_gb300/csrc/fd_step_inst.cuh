@@ -4,6 +4,7 @@
 #pragma once
 
 #include "fd_step.cuh"
+#include "fd_brick.cuh"
 #if FD_R == 2 || FD_R == 4
 #include "fd_tblock.cuh"
 #endif
@@ -34,7 +35,7 @@ cudaError_t set_smem_attr() {
   return e;
 }
 
-// The scheduled sweep (every mode but per-cell weights): the same shared
+// The scheduled sweep: the same shared
 // memory and launch bounds as the equal-share kernel, so the same CTAs fit on
 // an SM.
 template <int R, int TX, int TY, int PF, int MODE>
@@ -52,23 +53,17 @@ cudaError_t set_sched_smem_attr() {
 
 template <int R, int TX, int TY, int PF, int MODE>
 cudaError_t launch_one(const ShotDesc* shots, const long long* prefix, int nshots,
-                       const StepOverride& ov, int grid, cudaStream_t s) {
+                       const StepOverride& ov, int grid, bool pdl, cudaStream_t s) {
   if (ov.items) {
-    if constexpr (MODE != kModePerCell) {
-      cudaError_t e = set_sched_smem_attr<R, TX, TY, PF, MODE>();
-      if (e != cudaSuccess) return e;
-      sched_kernel<R, TX, TY, PF, MODE><<<grid, TX * TY, sweep_smem<R, TX, TY, PF, MODE>(), s>>>(
-          shots, ov);
-      return cudaGetLastError();
-    } else {
-      return cudaErrorInvalidValue;
-    }
+    cudaError_t e = set_sched_smem_attr<R, TX, TY, PF, MODE>();
+    if (e != cudaSuccess) return e;
+    return launch_step(sched_kernel<R, TX, TY, PF, MODE>, dim3(grid), TX * TY,
+                       sweep_smem<R, TX, TY, PF, MODE>(), pdl, s, shots, ov);
   }
   cudaError_t e = set_smem_attr<R, TX, TY, PF, MODE>();
   if (e != cudaSuccess) return e;
-  sweep_kernel<R, TX, TY, PF, MODE><<<grid, TX * TY, sweep_smem<R, TX, TY, PF, MODE>(), s>>>(
-      shots, prefix, nshots, ov);
-  return cudaGetLastError();
+  return launch_step(sweep_kernel<R, TX, TY, PF, MODE>, dim3(grid), TX * TY,
+                     sweep_smem<R, TX, TY, PF, MODE>(), pdl, s, shots, prefix, nshots, ov);
 }
 
 template <int R, int TX, int TY, int PF, int MODE>
@@ -101,10 +96,10 @@ int occupancy_one() {
 #define FD_PERCELL_LAUNCH(TX, TY)                                                          \
   case kModePerCell:                                                                       \
     return launch_one<FD_R, TX, TY, pf_of<FD_R, TX, TY, FD_MODE_PERCELL>(), FD_MODE_PERCELL>( \
-        shots, prefix, nshots, ov, grid, s);                                               \
+        shots, prefix, nshots, ov, grid, pdl, s);                                               \
   case kModeTable:                                                                         \
     return launch_one<FD_R, TX, TY, pf_of<FD_R, TX, TY, FD_MODE_TABLE>(), FD_MODE_TABLE>(     \
-        shots, prefix, nshots, ov, grid, s);
+        shots, prefix, nshots, ov, grid, pdl, s);
 #define FD_PERCELL_OCC(TX, TY)                                                                \
   case kModePerCell:                                                                          \
     return occupancy_one<FD_R, TX, TY, pf_of<FD_R, TX, TY, FD_MODE_PERCELL>(), FD_MODE_PERCELL>(); \
@@ -115,16 +110,16 @@ int occupancy_one() {
 template <>
 cudaError_t launch_sweep_r<FD_R>(const TileShape& t, int mode, const ShotDesc* shots,
                                  const long long* prefix, int nshots, const StepOverride& ov,
-                                 int grid, cudaStream_t s) {
+                                 int grid, bool pdl, cudaStream_t s) {
 #define FD_SHAPE(TX, TY)                                                                  \
   if (t.tx == TX && t.ty == TY) {                                                         \
     switch (mode) {                                                                       \
       case kModeForward:                                                                  \
-        return launch_one<FD_R, TX, TY, FD_PF(TX, TY), 0>(shots, prefix, nshots, ov, grid, s); \
+        return launch_one<FD_R, TX, TY, FD_PF(TX, TY), 0>(shots, prefix, nshots, ov, grid, pdl, s); \
       case kModeStoreE:                                                                   \
-        return launch_one<FD_R, TX, TY, FD_PF(TX, TY), 1>(shots, prefix, nshots, ov, grid, s); \
+        return launch_one<FD_R, TX, TY, FD_PF(TX, TY), 1>(shots, prefix, nshots, ov, grid, pdl, s); \
       case kModeAdjoint:                                                                  \
-        return launch_one<FD_R, TX, TY, FD_PF(TX, TY), 2>(shots, prefix, nshots, ov, grid, s); \
+        return launch_one<FD_R, TX, TY, FD_PF(TX, TY), 2>(shots, prefix, nshots, ov, grid, pdl, s); \
       FD_PERCELL_LAUNCH(TX, TY)                                                           \
       default: return cudaErrorInvalidValue;                                              \
     }                                                                                     \
@@ -149,6 +144,44 @@ int sweep_blocks_per_sm_r<FD_R>(const TileShape& t, int mode) {
   FD_FOR_EACH_SHAPE(FD_SHAPE)
 #undef FD_SHAPE
   return 0;
+}
+
+namespace {
+template <int R, int MODE>
+cudaError_t launch_brick_one(const ShotDesc* shot, const StepOverride& ov, dim3 grid, bool pdl,
+                             cudaStream_t s) {
+  static unsigned long long done = 0;  // one bit per device
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!(done & (1ull << (dev & 63)))) {
+    cudaError_t e = cudaFuncSetAttribute(brick_kernel<R, MODE>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         BrickCfg<R, MODE>::SMEM);
+    if (e != cudaSuccess) return e;
+    done |= 1ull << (dev & 63);
+  }
+  return launch_step(brick_kernel<R, MODE>, grid, BrickCfg<R, MODE>::NT, BrickCfg<R, MODE>::SMEM, pdl, s,
+                     shot, ov);
+}
+}  // namespace
+
+template <>
+cudaError_t launch_brick_r<FD_R>(int mode, const ShotDesc* shot, const StepOverride& ov, int Nx,
+                                 int Ny, int Nz, bool pdl, cudaStream_t s) {
+  using C = BrickCfg<FD_R, kModeForward>;
+  static_assert(C::TX == kBrickTile.tx && C::TY == kBrickTile.ty && C::ZB == kBrickPlanes,
+                "the tables and tensor maps are built for kBrickTile");
+  const dim3 grid((Nx + C::BX - 1) / C::BX, (Ny + C::BY - 1) / C::BY, (Nz + C::ZB - 1) / C::ZB);
+  switch (mode) {
+    case kModeForward: return launch_brick_one<FD_R, kModeForward>(shot, ov, grid, pdl, s);
+    case kModeStoreE: return launch_brick_one<FD_R, kModeStoreE>(shot, ov, grid, pdl, s);
+    case kModeAdjoint: return launch_brick_one<FD_R, kModeAdjoint>(shot, ov, grid, pdl, s);
+#if FD_R == 4
+    case kModePerCell: return launch_brick_one<FD_R, kModePerCell>(shot, ov, grid, pdl, s);
+    case kModeTable: return launch_brick_one<FD_R, kModeTable>(shot, ov, grid, pdl, s);
+#endif
+  }
+  return cudaErrorInvalidValue;
 }
 
 #if FD_R == 2 || FD_R == 4
