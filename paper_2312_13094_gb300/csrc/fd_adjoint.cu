@@ -139,14 +139,13 @@ fd_status adjoint_impl(fd_grid g, const fd_points* src, const float* wavelet,
     }
     if ((st = run_steps(g, rs))) return st;
   }
-  if ((st = check_device_error(g))) return st;
+  if ((st = check_run(g, drec, size_t(nt) * nrec))) return st;
 
   // ---- residual -------------------------------------------------------------
   float* dres = static_cast<float*>(g->resid.p);
   double* dloss = reinterpret_cast<double*>(static_cast<char*>(g->resid.p) +
                                             ((size_t(nt) * nrec * 4 + 15) / 16) * 16);
   if (nrec) {
-    if ((st = check_finite(g, drec, size_t(nt) * nrec))) return st;
     if (d_obs) {
       const float* dobs = nullptr;
       if ((st = stage_in(g, g->stage_aux, d_obs, size_t(nt) * nrec, &dobs))) return st;

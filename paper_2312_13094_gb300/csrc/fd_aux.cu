@@ -151,8 +151,7 @@ cudaError_t model_to_A(const float* data, int kind, int nx, int ny, int nz, int 
   return cudaGetLastError();
 }
 
-cudaError_t count_nonfinite(const float* x, size_t n, int* dcnt, int* hcnt,
-                            cudaStream_t s) {
+cudaError_t count_nonfinite_async(const float* x, size_t n, int* dcnt, cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(dcnt, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   if (n) {
@@ -160,6 +159,13 @@ cudaError_t count_nonfinite(const float* x, size_t n, int* dcnt, int* hcnt,
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
+  return cudaSuccess;
+}
+
+cudaError_t count_nonfinite(const float* x, size_t n, int* dcnt, int* hcnt,
+                            cudaStream_t s) {
+  cudaError_t e = count_nonfinite_async(x, n, dcnt, s);
+  if (e != cudaSuccess) return e;
   e = cudaMemcpyAsync(hcnt, dcnt, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return e;
   return cudaStreamSynchronize(s);

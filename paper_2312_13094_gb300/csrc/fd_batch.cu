@@ -367,9 +367,8 @@ extern "C" fd_status fd_batch_forward(int32_t nshots, const fd_shot* shots, int3
     // every grid's error word and receivers were written on stream s
     cudaStream_t own = g->stream;
     g->stream = s;
-    st = check_device_error(g);
     const int nrec = shots[i].rec ? shots[i].rec->n : 0;
-    if (!st && nrec) st = check_finite(g, P.drec[i], size_t(nt) * nrec);
+    st = check_run(g, P.drec[i], size_t(nt) * nrec);
     if (!st && nrec) st = finish_out(g, shots[i].rec_out, P.drec[i], size_t(nt) * nrec);
     g->stream = own;
     if (st) return st;

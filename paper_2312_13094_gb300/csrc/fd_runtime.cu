@@ -465,9 +465,8 @@ fd_status upload_tables(fd_grid g, const fd_points* src, double src_scale,
   if ((st = upload(g, t.recs, re))) return st;
   t.n_inj = int(ie.size());
   t.n_rec = int(re.size());
-  // keep the uploads ordered before the host vectors go away
-  cudaError_t e = cudaStreamSynchronize(g->stream);
-  if (e) return cuda_fail(e, "table upload");
+  // (an asynchronous copy from pageable memory has read it when it returns, so
+  // the vectors may go away)
   return FD_OK;
 }
 
@@ -940,6 +939,22 @@ fd_status check_finite(fd_grid g, const float* dev, size_t n) {
   return FD_OK;
 }
 
+// The error word of a finished run and the finite check of its n receiver
+// samples, with one wait and one read for both.
+fd_status check_run(fd_grid g, const float* rec, size_t n) {
+  int h[2] = {0, 0};
+  cudaError_t e = count_nonfinite_async(rec, n, g->d_err + 1, g->stream);
+  if (!e) e = cudaMemcpyAsync(h, g->d_err, sizeof(h), cudaMemcpyDeviceToHost, g->stream);
+  if (!e) e = cudaStreamSynchronize(g->stream);
+  if (e) return cuda_fail(e, "run check");
+  if (h[0]) {
+    cudaMemset(g->d_err, 0, sizeof(int));
+    return fail(FD_ERR_TIMEOUT, "a device-side wait ran out (error word %d)", h[0]);
+  }
+  if (h[1]) return fail(FD_ERR_NONFINITE, "%d receiver samples are NaN or Inf", h[1]);
+  return FD_OK;
+}
+
 // Copy between the padded pitched wavefield and a dense caller array.
 fd_status copy_field(fd_grid g, float* dev_field, void* user, int region, bool to_user) {
   cudaMemcpy3DParms p;
@@ -1194,13 +1209,12 @@ static fd_status propagate_impl(fd_grid g, int32_t n0, int32_t nsteps, const fd_
   }
   if ((st = run_steps(g, rs))) return st;
   }
-  if ((st = check_device_error(g))) return st;
-  if (nrec) {
-    if ((st = check_finite(g, drec, size_t(nsteps) * nrec))) return st;
+  if ((st = check_run(g, drec, size_t(nsteps) * nrec))) return st;
+  if (nrec && rec_out != drec) {
     if ((st = finish_out(g, rec_out, drec, size_t(nsteps) * nrec))) return st;
+    cudaError_t e = cudaStreamSynchronize(g->stream);
+    if (e) return cuda_fail(e, "stream synchronize");
   }
-  cudaError_t e = cudaStreamSynchronize(g->stream);
-  if (e) return cuda_fail(e, "stream synchronize");
   return FD_OK;
 }
 

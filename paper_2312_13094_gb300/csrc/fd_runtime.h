@@ -210,6 +210,7 @@ fd_status run_steps(fd_grid g, const RunSpec& rs);
 int grid_schedule(fd_grid g, int mode, StepOverride* ov, fd_status* st);
 fd_status check_device_error(fd_grid g);
 fd_status check_finite(fd_grid g, const float* dev, size_t n);
+fd_status check_run(fd_grid g, const float* rec, size_t n);  // both, with one wait
 fd_status copy_field(fd_grid g, float* dev_field, void* user, int region, bool to_user);
 // decomposed runs (fd_decomp.cu): steps of fd_forward / fd_propagate when the
 // grid has slabs, and the release of the slabs with the grid
