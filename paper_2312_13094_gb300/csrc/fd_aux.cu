@@ -24,11 +24,16 @@ __global__ void k_model_stats(const float* __restrict__ data, size_t n, int kind
     lo = fminf(lo, v);
     hi = fmaxf(hi, v);
   }
-  // positive floats order like their bit patterns
+  // positive floats order like their bit patterns; one atomic per warp (one
+  // per thread queued 2.6e5 of them on each word)
+  const unsigned lo_bits = __reduce_min_sync(0xffffffffu, __float_as_uint(lo));
+  const unsigned hi_bits = __reduce_max_sync(0xffffffffu, __float_as_uint(hi));
+  nbad = __reduce_add_sync(0xffffffffu, nbad);
+  if ((threadIdx.x & 31) != 0) return;
   if (nbad) atomicAdd(bad, nbad);
-  if (hi > 0.0f) {
-    atomicMin(vmin_bits, __float_as_uint(lo));
-    atomicMax(vmax_bits, __float_as_uint(hi));
+  if (hi_bits) {
+    atomicMin(vmin_bits, lo_bits);
+    atomicMax(vmax_bits, hi_bits);
   }
 }
 
@@ -83,14 +88,28 @@ __global__ void k_fold_grad(const float* __restrict__ gpad, int nx, int ny, int 
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   const int z = blockIdx.z;
-  if (x >= nx) return;
   const int xa = x == 0 ? 0 : x + nbl, xb = x == nx - 1 ? Nx - 1 : x + nbl;
   const int ya = y == 0 ? 0 : y + nbl, yb = y == ny - 1 ? Ny - 1 : y + nbl;
   const int za = z == 0 ? 0 : z + nbl, zb = z == nz - 1 ? Nz - 1 : z + nbl;
   double acc = 0.0;
-  for (int k = za; k <= zb; ++k)
-    for (int j = ya; j <= yb; ++j)
-      for (int i = xa; i <= xb; ++i) acc += gpad[((size_t)k * Ny + j) * pitch + i];
+  // the columns of an x end (nbl + 1 cells or more per row) over the lanes of
+  // its warp, rows in turn: a corner alone sums (nbl + 1)^3 cells
+  const bool end = x < nx && xb > xa;
+  for (unsigned todo = __ballot_sync(0xffffffffu, end); todo; todo &= todo - 1) {
+    const int src = __ffs(todo) - 1, lane = threadIdx.x & 31;
+    const int a = __shfl_sync(0xffffffffu, xa, src), w = __shfl_sync(0xffffffffu, xb, src) - a + 1;
+    const int rows = yb - ya + 1;
+    double part = 0.0;
+    for (int k = za; k <= zb; ++k)
+      for (int e = lane; e < rows * w; e += 32)
+        part += gpad[((size_t)k * Ny + ya + e / w) * pitch + a + e % w];
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (lane == src) acc = part;
+  }
+  if (x >= nx) return;
+  if (!end)
+    for (int k = za; k <= zb; ++k)
+      for (int j = ya; j <= yb; ++j) acc += gpad[((size_t)k * Ny + j) * pitch + xa];
   gphys[((size_t)z * ny + y) * nx + x] = (float)acc;
 }
 
@@ -127,7 +146,7 @@ cudaError_t model_stats(const float* data, size_t n, int kind, float* vmin,
   unsigned int init[3] = {0x7f800000u, 0u, 0u};
   cudaError_t e = cudaMemcpyAsync(scratch, init, sizeof(init), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  k_model_stats<<<1024, 256, 0, s>>>(data, n, kind, scratch, scratch + 1,
+  k_model_stats<<<304, 256, 0, s>>>(data, n, kind, scratch, scratch + 1,
                                      reinterpret_cast<int*>(scratch + 2));
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;

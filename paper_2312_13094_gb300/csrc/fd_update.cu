@@ -13,12 +13,19 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "fd_aux.h"
 #include "fd_runtime.h"
 
 namespace fd {
 namespace {
+
+// Scratch of the maxima: one of kSlots device words (four each) per call in
+// flight, so that a step allocates nothing; further concurrent calls allocate.
+constexpr int kSlots = 16;
+__device__ unsigned int g_scratch[kSlots][4];
+std::atomic<bool> g_taken[kSlots];
 
 __global__ void k_absmax2(const float* __restrict__ m, const float* __restrict__ g, size_t n,
                           unsigned int* out) {
@@ -80,8 +87,20 @@ extern "C" fd_status fd_descent_step(int64_t n, float* m, const float* grad, dou
     return fail(FD_ERR_ARG, "fd_descent_step takes device arrays only");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   unsigned int* scratch = nullptr;
-  cudaError_t e = dev_alloc(reinterpret_cast<void**>(&scratch), 4 * sizeof(unsigned int));
-  if (e) return cuda_fail(e, "update scratch allocation");
+  cudaError_t e = cudaSuccess;
+  int slot = 0;
+  while (slot < kSlots && g_taken[slot].exchange(true)) ++slot;
+  if (slot < kSlots) {
+    void* base = nullptr;
+    e = cudaGetSymbolAddress(&base, g_scratch);  // of the current device
+    scratch = static_cast<unsigned int*>(base) + 4 * slot;
+  } else {
+    e = dev_alloc(reinterpret_cast<void**>(&scratch), 4 * sizeof(unsigned int));
+  }
+  if (e) {
+    if (slot < kSlots) g_taken[slot] = false;
+    return cuda_fail(e, "update scratch allocation");
+  }
   unsigned int h[4] = {0, 0, 0, 0};
   const int nb = blocks_for(size_t(n));
   e = cudaMemsetAsync(scratch, 0, sizeof(h), s);
@@ -112,6 +131,10 @@ extern "C" fd_status fd_descent_step(int64_t n, float* m, const float* grad, dou
     }
     if (!st && alpha_out) *alpha_out = alpha;
   }
-  cudaFree(scratch);
+  // (the stream has been waited for: nothing reads the words any more)
+  if (slot < kSlots)
+    g_taken[slot] = false;
+  else
+    cudaFree(scratch);
   return st;
 }
