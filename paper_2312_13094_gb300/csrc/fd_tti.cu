@@ -155,31 +155,43 @@ __global__ void k_tti_stats(const float* __restrict__ vp, const float* __restric
   }
 }
 
-// rec[row][r] = sum_k w_k p[off_k]
-__global__ void k_tti_gather(const float2* __restrict__ u, const TtiRec* __restrict__ recs, int n,
-                             float* __restrict__ out) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  const TtiRec e = recs[r];
-  float acc = 0.f;
+// The points between two steps, on u = (p, q)^n: first the sources of the step
+// that made u,
+//   p, q at each source node += A w q(t_{n-1}) / (h (1 + b))
+// (s^n = w q / h^3 scaled by dt^2 v^2 and the damping division of the update;
+// val null: none), then the receivers, rec[n][r] = sum_k w_k p[off_k] (out null:
+// none).  Both in one launch take one block, so that the receivers see the sources.
+constexpr int kPointThreads = 512, kPointsAtOnce = 4096;
+__global__ void __launch_bounds__(kPointThreads)
+    k_tti_points(const TtiInj* __restrict__ inj, int ninj, const float* __restrict__ val,
+                 const float2* __restrict__ coef, float bscale, int nbl, int nx, int ny, int nz,
+                 float2* u, const TtiRec* __restrict__ recs, int nrec, float* __restrict__ out) {
+  pdl_trigger();
+  pdl_wait();
+  if (val) {
+    for (int i = blockIdx.x * kPointThreads + threadIdx.x; i < ninj;
+         i += gridDim.x * kPointThreads) {
+      const TtiInj e = inj[i];
+      const int dx = depth(e.x, nbl, nx), dy = depth(e.y, nbl, ny), dz = depth(e.z, nbl, nz);
+      const float b = bscale * static_cast<float>(dx * dx + dy * dy + dz * dz);
+      const float s = coef[e.off].x * e.w * val[e.col] / (1.f + b);
+      atomicAdd(&u[e.off].x, s);
+      atomicAdd(&u[e.off].y, s);
+    }
+    __threadfence();
+    __syncthreads();
+  }
+  if (out) {
+    for (int r = blockIdx.x * kPointThreads + threadIdx.x; r < nrec;
+         r += gridDim.x * kPointThreads) {
+      const TtiRec e = recs[r];
+      float acc = 0.f;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc = fmaf(e.w[k], u[e.off[k]].x, acc);
-  out[r] = acc;
-}
-
-// p, q at each source node += A w q(t_n) / (h (1 + b)) (s^n = w q / h^3 scaled
-// by dt^2 v^2 and the damping division of the update)
-__global__ void k_tti_inject(const TtiInj* __restrict__ inj, int n, const float* __restrict__ val,
-                             const float2* __restrict__ coef, float bscale, int nbl, int nx, int ny,
-                             int nz, float2* u) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const TtiInj e = inj[i];
-  const int dx = depth(e.x, nbl, nx), dy = depth(e.y, nbl, ny), dz = depth(e.z, nbl, nz);
-  const float b = bscale * static_cast<float>(dx * dx + dy * dy + dz * dz);
-  const float s = coef[e.off].x * e.w * val[e.col] / (1.f + b);
-  atomicAdd(&u[e.off].x, s);
-  atomicAdd(&u[e.off].y, s);
+      for (int k = 0; k < 8; ++k)  // (L2: where the atomics went)
+        acc = fmaf(e.w[k], __ldcg(&u[e.off[k]].x), acc);
+      out[r] = acc;
+    }
+  }
 }
 
 // Rows [row0, row0 + rows) of the padded grid (row = z Ny + y) between the
@@ -199,7 +211,8 @@ __global__ void k_tti_field(float2* __restrict__ u, float* __restrict__ dense, i
 
 // Launches one step on the resident CTAs (*ctas, found by the first call).
 template <int R>
-cudaError_t launch_q(const tti::QMaps& M, const tti::QArgs& qa, int* ctas, cudaStream_t s) {
+cudaError_t launch_q(const tti::QMaps& M, const tti::QArgs& qa, int* ctas, bool pdl,
+                     cudaStream_t s) {
   if (*ctas == 0) {
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -211,27 +224,26 @@ cudaError_t launch_q(const tti::QMaps& M, const tti::QArgs& qa, int* ctas, cudaS
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, tti::k_tti_q<R>, tti::kQT,
                                                         tti::QGeom<R>::SMEM);
     if (e) return e;
-    // at least 2R planes per share: each run of planes first enters 2R
+    // at least R planes per share: each run of planes first enters 2R
     const long long units = (long long)qa.cols * qa.Nz;
     *ctas = int(std::max<long long>(
-        1, std::min<long long>((long long)std::max(per, 1) * sms, units / (2 * R))));
+        1, std::min<long long>((long long)std::max(per, 1) * sms, units / R)));
   }
-  tti::k_tti_q<R><<<*ctas, tti::kQT, tti::QGeom<R>::SMEM, s>>>(M, qa);
-  return cudaGetLastError();
+  return launch_step(tti::k_tti_q<R>, dim3(*ctas), tti::kQT, tti::QGeom<R>::SMEM, pdl, s, M, qa);
 }
 
-cudaError_t launch_q_r(int R, const tti::QMaps& M, const tti::QArgs& qa, int* ctas,
+cudaError_t launch_q_r(int R, const tti::QMaps& M, const tti::QArgs& qa, int* ctas, bool pdl,
                        cudaStream_t s) {
   count_launch();
   switch (R) {
-    case 1: return launch_q<1>(M, qa, ctas, s);
-    case 2: return launch_q<2>(M, qa, ctas, s);
-    case 3: return launch_q<3>(M, qa, ctas, s);
-    case 4: return launch_q<4>(M, qa, ctas, s);
-    case 5: return launch_q<5>(M, qa, ctas, s);
-    case 6: return launch_q<6>(M, qa, ctas, s);
-    case 7: return launch_q<7>(M, qa, ctas, s);
-    case 8: return launch_q<8>(M, qa, ctas, s);
+    case 1: return launch_q<1>(M, qa, ctas, pdl, s);
+    case 2: return launch_q<2>(M, qa, ctas, pdl, s);
+    case 3: return launch_q<3>(M, qa, ctas, pdl, s);
+    case 4: return launch_q<4>(M, qa, ctas, pdl, s);
+    case 5: return launch_q<5>(M, qa, ctas, pdl, s);
+    case 6: return launch_q<6>(M, qa, ctas, pdl, s);
+    case 7: return launch_q<7>(M, qa, ctas, pdl, s);
+    case 8: return launch_q<8>(M, qa, ctas, pdl, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -419,25 +431,43 @@ fd_status propagate(fd_tti t, int n0, int nsteps, const fd_points* src, const fl
   qa.cols_y = (t->Ny + tti::kQY - 1) / tti::kQY;
   qa.cols = qa.cols_y * ((t->Nx + tti::kQX - 1) / tti::kQX);
   if (t->profiling) cudaEventRecord(t->ev0, t->stream);
+  // Launches of short steps may start before the one ahead has finished (us a
+  // step without / with it, points in their own launches before: 68^3 SO 8
+  // 20.6 / 16.9, 24.5; 100^3 SO 16 51.0 / 45.5, 55.0; 243 x 181 x 207 SO 16 221 / 216).
+  // Long steps lose by it (336^3 SO 8 469 / 499; 200^3 SO 4 94 / 102).
+  const bool early =
+      (long long)t->Nx * t->Ny * t->Nz <= (t->R <= 4 ? 4000000LL : 16000000LL);
+  // sources of step `s` (-1: none) and receivers of the field it made, on u;
+  // many of them in two launches of several blocks
+  auto points = [&](int s, float2* u, bool first) -> cudaError_t {
+    const bool inj = t->n_inj && s >= 0, rec = nrec && s + 1 < nsteps;
+    const float* val = inj ? dval + size_t(n0 + s) * nsrc : nullptr;
+    float* out = rec ? drec + size_t(s + 1) * nrec : nullptr;
+    auto launch = [&](int blocks, const float* v, float* o) {
+      count_launch();
+      return launch_step(k_tti_points, dim3(blocks), kPointThreads, 0, early && !first, t->stream,
+                         static_cast<const TtiInj*>(t->inj.p), t->n_inj, v, t->coef, t->bscale,
+                         t->d.nbl, t->d.nx, t->d.ny, t->d.nz, u,
+                         static_cast<const TtiRec*>(t->rec.p), nrec, o);
+    };
+    auto blocks = [](int n) { return (n + kPointThreads - 1) / kPointThreads; };
+    if (!inj && !rec) return cudaSuccess;
+    if (t->n_inj <= kPointsAtOnce && nrec <= kPointsAtOnce) return launch(1, val, out);
+    cudaError_t er = inj ? launch(blocks(t->n_inj), val, nullptr) : cudaSuccess;
+    if (!er && rec) er = launch(blocks(nrec), nullptr, out);
+    return er;
+  };
+  if ((e = points(-1, t->u[t->cur], true))) return cuda_fail(e, "TTI points launch");
   for (int s = 0; s < nsteps; ++s) {
     const int cur = t->cur;
-    if (nrec) {
-      k_tti_gather<<<(nrec + 127) / 128, 128, 0, t->stream>>>(
-          t->u[cur], static_cast<const TtiRec*>(t->rec.p), nrec, drec + size_t(s) * nrec);
-      count_launch();
-    }
     tti::QMaps M;
     M.halo = t->halo[cur];
     M.prev = t->tile[cur ^ 1];
     M.coef = t->coef_map;
     qa.out = t->u[cur ^ 1];
-    if ((e = launch_q_r(t->R, M, qa, &t->ctas, t->stream))) return cuda_fail(e, "TTI step launch");
-    if (t->n_inj) {
-      k_tti_inject<<<(t->n_inj + 127) / 128, 128, 0, t->stream>>>(
-          static_cast<const TtiInj*>(t->inj.p), t->n_inj, dval + size_t(n0 + s) * nsrc, t->coef,
-          t->bscale, t->d.nbl, t->d.nx, t->d.ny, t->d.nz, t->u[cur ^ 1]);
-      count_launch();
-    }
+    if ((e = launch_q_r(t->R, M, qa, &t->ctas, early && s > 0, t->stream)))
+      return cuda_fail(e, "TTI step launch");
+    if ((e = points(s, t->u[cur ^ 1], false))) return cuda_fail(e, "TTI points launch");
     t->cur = cur ^ 1;
   }
   if (t->profiling) {

@@ -180,6 +180,8 @@ __global__ void __launch_bounds__(kQT, q_ctas(R))
   const long long hi = units * (blockIdx.x + 1) / gridDim.x;
   bool bad = false;
   long long limit = a.spin_limit;
+  pdl_trigger();
+  pdl_wait();
 
   for (int w = 0; w < waves || pos < hi; ++w) {
     int col = w * gridDim.x + blockIdx.x, z0 = 0, z1 = a.Nz;
