@@ -43,9 +43,12 @@ struct BrickCfg {
   static constexpr int CTAS =
       R <= 3 ? 4 : (R == 4 && MODE != kModePerCell ? 3 : (R <= 7 ? 2 : 1));
   static_assert(CTAS * (SMEM + 1024) <= 228 * 1024, "resident CTAs");
-  static constexpr int NCOPY = NP + (2 + NC) * ZB;
   static_assert(TBYTES % 128 == 0, "tile pitch");
 };
+
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* m) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
+}
 
 template <int R, int MODE>
 __global__ void __launch_bounds__(BrickCfg<R, MODE>::NT, BrickCfg<R, MODE>::CTAS)
@@ -61,39 +64,37 @@ __global__ void __launch_bounds__(BrickCfg<R, MODE>::NT, BrickCfg<R, MODE>::CTAS
   const StepArgs& a = shot->args;
   const int cur = ov.cur;
   pdl_trigger();
+  if (tid < 3)  // the tensor maps, fetched while the step ahead still runs
+    prefetch_map(tid == 0 ? &shot->halo[cur] : (tid == 1 ? &shot->tile[cur ^ 1] : &shot->A));
   if (tid == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
+    mbar_expect_tx(bar, C::NP * C::UBYTES + (2 + C::NC) * C::ZB * C::TBYTES);
   }
   if (MODE == kModeTable)  // (written before the first step)
     for (int i = tid; i < 2 * a.tab_nodes; i += C::NT) tab[i] = a.table[i];
-  pdl_wait();
-  // once a wait of this run has failed, later launches return at once (the
-  // word is read by every thread behind the barrier of an earlier launch's end:
-  // the launch before this one wrote it, or nobody)
-  __shared__ int s_abort;
-  if (tid == 0) s_abort = *reinterpret_cast<volatile const int*>(a.err);
   __syncthreads();
-  if (s_abort) return;
-  if (tid == 0) mbar_expect_tx(bar, C::NP * C::UBYTES + (2 + C::NC) * C::ZB * C::TBYTES);
-  __syncwarp();
-  if (tid < 32) {  // the copies over the lanes of warp 0
+  // the copies over the lanes of warp 0: A and the coefficients, which no step
+  // writes, before the step ahead has finished, the wavefields after it
+  if (tid < C::ZB)
+    tma_load_3d(sbase + C::OFF_A + tid * C::TBYTES, &shot->A, x0, y0, zb + tid, bar);
+  if (tid < 32) {
 #pragma unroll
-    for (int c = tid; c < C::NCOPY; c += 32) {
+    for (int c = tid; c < C::NC * C::ZB; c += 32)  // field j sits j * Nz planes further
+      tma_load_3d(sbase + C::OFF_C + c * C::TBYTES, &shot->C, x0, y0,
+                  zb + c % C::ZB + c / C::ZB * a.Nz, bar);
+  }
+  pdl_wait();
+  if (tid < 32) {
+#pragma unroll
+    for (int c = tid; c < C::NP + C::ZB; c += 32) {
       if (c < C::NP) {
         const int z = zb - R + c;
         if (ov.debug_skip_plane < 0 || z != ov.debug_skip_plane)
           tma_load_3d(sbase + c * C::UPITCH, &shot->halo[cur], x0 - C::RX, y0 - R, z, bar);
-      } else if (c < C::NP + C::ZB) {
+      } else {
         const int i = c - C::NP;
         tma_load_3d(sbase + C::OFF_P + i * C::TBYTES, &shot->tile[cur ^ 1], x0, y0, zb + i, bar);
-      } else if (c < C::NP + 2 * C::ZB) {
-        const int i = c - C::NP - C::ZB;
-        tma_load_3d(sbase + C::OFF_A + i * C::TBYTES, &shot->A, x0, y0, zb + i, bar);
-      } else {  // coefficient field j sits j * Nz planes further
-        const int i = c - C::NP - 2 * C::ZB;
-        tma_load_3d(sbase + C::OFF_C + i * C::TBYTES, &shot->C, x0, y0,
-                    zb + i % C::ZB + i / C::ZB * a.Nz, bar);
       }
     }
   }
@@ -144,12 +145,16 @@ __global__ void __launch_bounds__(BrickCfg<R, MODE>::NT, BrickCfg<R, MODE>::CTAS
   const int zf_lo = no_sponge ? 0 : a.nbl, zf_hi = no_sponge ? Nz : a.nbl + a.nz;
   const bool ok[4] = {gx < a.xend, gx + 1 < a.xend, gx + 2 < a.xend, gx + 3 < a.xend};
 
+  // once a wait of this run has failed, its later launches do nothing; the word
+  // is read while the copies are on their way, and they are waited for either way
+  const bool failed = *reinterpret_cast<volatile const int*>(a.err) != 0;
   // every thread waits, so that each sees the copies; on expiry (the copies
   // of this CTA have then had the whole limit to land) the CTA records it
   if (!mbar_wait(bar, 0, ov.spin_limit)) {
     atomicOr(a.err, 1);
     return;
   }
+  if (failed) return;
 
   const uint32_t crow = 4u * ((ty + R) * C::W + 4 * tx + C::RX);
   const uint32_t own = sbase + C::ZT * zg * C::UPITCH + crow;  // plane k0 - R
