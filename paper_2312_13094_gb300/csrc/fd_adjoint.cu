@@ -43,6 +43,17 @@ fd_status copy_async(fd_grid g, void* dst, const void* src, size_t bytes) {
   return FD_OK;
 }
 
+// Puts a grid's forward wavefields (and their tensor maps) back, with the
+// current buffer as the last run left it.
+struct FieldsGuard {
+  fd_grid g;
+  Fields f;
+  ~FieldsGuard() {
+    f.cur = g->F.cur;
+    g->F = f;
+  }
+};
+
 // Shared body of fd_adjoint_gradient (d_obs given) and fd_backward
 // (residual given).
 fd_status adjoint_impl(fd_grid g, const fd_points* src, const float* wavelet,
@@ -168,19 +179,24 @@ fd_status adjoint_impl(fd_grid g, const fd_points* src, const float* wavelet,
       return cuda_fail(e, "adjoint reset");
   g->Z.cur = 0;
   float* ebase = static_cast<float*>(g->ebuf.p);
+  FieldsGuard own{g, g->F};  // the grid's own wavefields, back in place on return
   for (int s = nseg - 1; s >= 0; --s) {
     const int n0 = s * L, n1 = std::min(nt, n0 + L);
-    // restore (u^{n0-1}, u^{n0}) and recompute the segment storing e^{n+1}
-    g->F.cur = 0;
+    // recompute the segment from (u^{n0-1}, u^{n0}), storing e^{n+1}: in the
+    // checkpoint's own memory, which nothing needs afterwards, or from rest in
+    // the grid's wavefields
     if (s == 0) {
+      g->F = own.f;
       for (int b = 0; b < 2; ++b)
         if ((e = cudaMemsetAsync(g->F.u[b], 0, cell_bytes, g->stream)))
           return cuda_fail(e, "wavefield reset");
     } else {
-      const char* slot = ck + size_t(s - 1) * 2 * cell_bytes;
-      if ((st = copy_async(g, g->F.u[1], slot, cell_bytes))) return st;
-      if ((st = copy_async(g, g->F.u[0], slot + cell_bytes, cell_bytes))) return st;
+      char* slot = ck + size_t(s - 1) * 2 * cell_bytes;
+      g->F.u[1] = reinterpret_cast<float*>(slot);
+      g->F.u[0] = reinterpret_cast<float*>(slot + cell_bytes);
+      if ((st = build_field_maps(g, g->F))) return st;
     }
+    g->F.cur = 0;
     RunSpec rf;
     memset(&rf, 0, sizeof(rf));
     rf.f = &g->F;
