@@ -47,12 +47,11 @@ struct TaylorC {
 // sums over units are shuffles.
 //
 // What bounds it: shared-memory reads (two 128-bit loads per 16 FMAs; the FMAs
-// alone, 14 336 per sample forward and backward, would take 23 us of the 61 us
+// alone, 14 336 per sample forward and backward, would take 23 us of the 60 us
 // below).  One thread per sample, the former layout, read one shared word per
 // FMA and kept four warps per SM; here 16 warps per SM share each operand.
 // Loss and gradient of 65 536 samples: 196 -> 83 us a call, of which the kernel
-// 61 us; per-cell weights of 230 x 213 x 181 cells with the shot that follows:
-// 18.1 -> 15.8 ms.
+// 60 us.
 //
 // Only s_j = (o_j + o_{j+4}) / 2 enters the coefficients, so o_j + o_{j+4} is
 // one sum and dL/do_j = dL/do_{j+4} is formed once.  (Adding the two weight rows
@@ -67,8 +66,7 @@ constexpr int NSUB = 8;       // samples per warp: the unit in which work is dea
 // only) W2 as stored, the activation tiles and two staged sample chunks.
 constexpr int SM_W1 = 0, SM_B1 = SM_W1 + 4 * H, SM_B2 = SM_B1 + H, SM_W3 = SM_B2 + H,
               SM_B3 = SM_W3 + NOUT * H, SM_W2T = SM_B3 + NOUT, SM_H1T = SM_W2T + H * H,
-              SM_FWD = SM_H1T + H * S,
-              SM_W2 = SM_FWD, SM_H1 = SM_W2 + H * H, SM_D2 = SM_H1 + S * H,
+              SM_W2 = SM_H1T + H * S, SM_H1 = SM_W2 + H * H, SM_D2 = SM_H1 + S * H,
               SM_D2T = SM_D2 + S * H, SM_SMP = SM_D2T + H * S,
               SM_GRAD = SM_SMP + 2 * S * SAMPLE;
 static_assert(SM_W2T % 4 == 0 && SM_SMP % 4 == 0, "float4 tiles");
@@ -87,30 +85,34 @@ __device__ __forceinline__ float at4(const float4& v, int i) {
 }
 
 // Parameters into shared memory: W1, W3, biases, W2 transposed (W2T[i][k]) and, to keep, W2 as stored.
+template <int T>
 __device__ __forceinline__ void load_params(float* sm, const float* __restrict__ p, bool keep) {
-  for (int i = threadIdx.x; i < 4 * H; i += NTHR) {
+  for (int i = threadIdx.x; i < 4 * H; i += T) {
     sm[SM_W1 + i] = p[OW1 + i];
     sm[SM_W3 + i] = p[OW3 + i];
     sm[SM_W3 + RL * H + i] = p[OW3 + RL * H + i];
   }
-  for (int i = threadIdx.x; i < H; i += NTHR) {
+  for (int i = threadIdx.x; i < H; i += T) {
     sm[SM_B1 + i] = p[OB1 + i];
     sm[SM_B2 + i] = p[OB2 + i];
   }
   if (threadIdx.x < NOUT) sm[SM_B3 + threadIdx.x] = p[OB3 + threadIdx.x];
-  // W2 by 4 x 4 blocks, transposed in registers (one block per thread)
-  static_assert(NTHR * 16 == H * H && OW2 % 4 == 0, "one block of W2 per thread");
-  const int kb = threadIdx.x & 15, ub = threadIdx.x >> 4;
-  float4 w[4];
+  // W2 by 4 x 4 blocks, transposed in registers
+  static_assert(OW2 % 4 == 0, "float4 rows of W2");
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    w[r] = *reinterpret_cast<const float4*>(p + OW2 + (4 * kb + r) * H + 4 * ub);
-    if (keep) *reinterpret_cast<float4*>(sm + SM_W2 + (4 * kb + r) * H + 4 * ub) = w[r];
+  for (int e = threadIdx.x; e < H * H / 16; e += T) {
+    const int kb = e & 15, ub = e >> 4;
+    float4 w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      w[r] = *reinterpret_cast<const float4*>(p + OW2 + (4 * kb + r) * H + 4 * ub);
+      if (keep) *reinterpret_cast<float4*>(sm + SM_W2 + (4 * kb + r) * H + 4 * ub) = w[r];
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      st4(sm + SM_W2T + (4 * ub + r) * H + 4 * kb, at4(w[0], r), at4(w[1], r), at4(w[2], r),
+          at4(w[3], r));
   }
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-    st4(sm + SM_W2T + (4 * ub + r) * H + 4 * kb, at4(w[0], r), at4(w[1], r), at4(w[2], r),
-        at4(w[3], r));
 }
 
 // acc[s][u] += a_s b_u
@@ -195,25 +197,41 @@ __device__ __forceinline__ float layer2_out(const float* sm, int sg, int ug, flo
 // of a grid, where x0 = v dt / h = sqrt(A) because A = dt^2 v^2 / h^2 and
 // coefficient field j lies at coef + j * n (columns x >= Nx get the Taylor
 // weights).
+//
+// A chunk of 128 samples on 128 threads as 8 x 8 register tiles: thread
+// (sg, ug) = (tid / 8, tid % 8) holds samples 8 sg .. 8 sg + 7 by units 4 ug ..
+// 4 ug + 3 and 32 + 4 ug .. 35 + 4 ug, so that a step reads four 128-bit words
+// per 64 FMAs, half as many as a 4 x 4 tile (there is no gradient to keep in
+// registers here; with it, 8 x 8 tiles leave eight warps per SM, and k_mlp_grad
+// took 70 us instead of 60).  230 x 213 x 181 cells: 2.25 -> 1.9 ms against 4 x 4
+// tiles, 1.1 ms of it FMAs.
 // ---------------------------------------------------------------------------
+constexpr int CS = 128, CTHR = 128;  // samples per chunk, threads
+constexpr int SM_CH1T = SM_W2T + H * H, SM_COEF = SM_CH1T + H * CS;
+
+// Float4 block h (of two) of sample group sg in row `row` of the [unit][sample]
+// tile, permuted so that eight unit groups writing it touch all banks.
+__device__ __forceinline__ int cblk(int row, int sg, int h) {
+  return row * CS + 4 * ((2 * sg + h) ^ ((row >> 2) & 7));
+}
+
 template <bool GRID>
-__global__ void __launch_bounds__(NTHR, 3)
+__global__ void __launch_bounds__(CTHR, 4)
     k_mlp_coef(const float* __restrict__ params, const float* __restrict__ in, size_t n, int pitch,
                int Nx, float x1, float x2, float x3, TaylorC t, float* __restrict__ coef) {
   extern __shared__ __align__(16) float sm[];
-  const int tid = threadIdx.x, sg = tid >> 4, ug = tid & 15, j = ug & 3;
-  load_params(sm, params, false);
+  const int tid = threadIdx.x, sg = tid >> 3, ug = tid & 7;
+  load_params<CTHR>(sm, params, false);
   __syncthreads();
-  const float tc = t.c[j + 1];
-  const size_t step = size_t(gridDim.x) * S;
+  const size_t step = size_t(gridDim.x) * CS;
   const int xstep = GRID ? int(step % pitch) : 0;
-  size_t base = size_t(blockIdx.x) * S;
-  int col = GRID ? int((base + 4 * sg + (ug >> 2)) % pitch) : 0;  // of the lane's own cell
+  size_t base = size_t(blockIdx.x) * CS;
+  int col = GRID ? int((base + tid) % pitch) : 0;  // of the lane's own cell
   for (; base < n; base += step) {
-    float x[4][NIN], h1[4][4], h2[4][4];
+    float x[8][NIN];
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      const size_t i = base + 4 * sg + s;
+    for (int s = 0; s < 8; ++s) {
+      const size_t i = base + 8 * sg + s;
       if (GRID) {
         x[s][0] = i < n ? sqrtf(in[i]) : 0.f;
         x[s][1] = x1;
@@ -225,16 +243,80 @@ __global__ void __launch_bounds__(NTHR, 3)
       }
     }
     __syncwarp();  // a warp's samples are written and read by the warp alone
-    layer1(sm, sg, ug, x, h1);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int k = (u >> 2) * 32 + 4 * ug + (u & 3);
+      const float4 w = ld4(sm + SM_W1 + 4 * k);
+      const float b = sm[SM_B1 + k];
+      float h[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        float z = b;
+#pragma unroll
+        for (int c = 0; c < NIN; ++c) z = fmaf(at4(w, c), x[s][c], z);
+        h[s] = fmaxf(z, 0.0f);
+      }
+      st4(sm + SM_CH1T + cblk(k, sg, 0), h[0], h[1], h[2], h[3]);
+      st4(sm + SM_CH1T + cblk(k, sg, 1), h[4], h[5], h[6], h[7]);
+    }
     __syncwarp();
-    const float sj = layer2_out(sm, sg, ug, h2);
-    const size_t i = base + 4 * sg + (ug >> 2);
-    if (i < n) {
-      const float c = tc * (1.0f + 0.5f * tanhf(sj));
-      if (GRID)
-        coef[j * n + i] = col < Nx ? c : tc;
-      else
-        coef[i * RL + j] = c;
+    float h2[8][8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+      for (int s = 0; s < 8; ++s) h2[s][u] = sm[SM_B2 + (u >> 2) * 32 + 4 * ug + (u & 3)];
+#pragma unroll 2
+    for (int r4 = 0; r4 < H / 4; ++r4) {
+      const float* t0 = sm + SM_CH1T + cblk(4 * r4, sg, 0);
+      const float* t1 = sm + SM_CH1T + cblk(4 * r4, sg, 1);
+      const float* w = sm + SM_W2T + 4 * r4 * H + 4 * ug;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float4 a[2] = {ld4(t0 + r * CS), ld4(t1 + r * CS)};
+        const float4 b[2] = {ld4(w + r * H), ld4(w + r * H + 32)};
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            h2[s][u] = fmaf(at4(a[s >> 2], s & 3), at4(b[u >> 2], u & 3), h2[s][u]);
+      }
+    }
+    // sums over units, reduced and scattered over the eight lanes: lane ug ends
+    // with the outputs of sample 8 sg + ug
+    auto fold = [&](float lo, float hi, int m) {
+      const bool up = (ug & m) != 0;
+      return (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, m);
+    };
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) h2[s][u] = fmaxf(h2[s][u], 0.0f);
+    const size_t i = base + tid;
+#pragma unroll
+    for (int j = 0; j < RL; ++j) {
+      float z[8];
+#pragma unroll
+      for (int s = 0; s < 8; ++s) z[s] = 0.f;
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const float4 w = ld4(sm + SM_W3 + j * H + 32 * hf + 4 * ug);
+        const float4 w4 = ld4(sm + SM_W3 + (j + RL) * H + 32 * hf + 4 * ug);
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            z[s] = fmaf(at4(w4, u), h2[s][4 * hf + u], fmaf(at4(w, u), h2[s][4 * hf + u], z[s]));
+      }
+      const float o = fold(fold(fold(z[0], z[4], 4), fold(z[2], z[6], 4), 2),
+                           fold(fold(z[1], z[5], 4), fold(z[3], z[7], 4), 2), 1);
+      const float sj = 0.5f * (o + (sm[SM_B3 + j] + sm[SM_B3 + RL + j]));
+      if (i < n) {
+        const float c = t.c[j + 1] * (1.0f + 0.5f * tanhf(sj));
+        if (GRID)
+          coef[j * n + i] = col < Nx ? c : t.c[j + 1];
+        else
+          coef[i * RL + j] = c;
+      }
     }
     if (GRID) {
       col += xstep;
@@ -283,7 +365,7 @@ __global__ void __launch_bounds__(NTHR, 2)
   };
   float nxt[NST];
   fetch(lo, nxt);
-  load_params(sm, params, true);
+  load_params<NTHR>(sm, params, true);
   const float tc = t.c[j + 1];
   float a1[4][4], a2[4][4], a3[4][4], ab1[4], ab2[4], ab3 = 0.f;
 #pragma unroll
@@ -539,6 +621,16 @@ TaylorC taylor_c() {
   return t;
 }
 
+// The inference kernels' dynamic shared memory, above the default limit.
+fd_status coef_attr() {
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_coef<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       int(SM_COEF * sizeof(float)));
+  if (!e)
+    e = cudaFuncSetAttribute(k_mlp_coef<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int(SM_COEF * sizeof(float)));
+  return e ? cuda_fail(e, "kernel attribute") : FD_OK;
+}
+
 int sm_count() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -560,7 +652,7 @@ struct fd_mlp_s {
   float* m = nullptr;   // Adam first moment
   float* v = nullptr;   // Adam second moment
   double* loss = nullptr;  // behind the gradient in its allocation
-  float* host = nullptr;    // pinned image of gradient and loss
+  std::vector<float> host;  // image of gradient and loss
   int t = 0;               // Adam step count
   DevBuf stage, stage2;
 };
@@ -571,9 +663,11 @@ fd_status mlp_grid_coefficients(fd_mlp net, const float* A, size_t ncell, int pi
                                 double h, double dt, double f_hz, float* coef,
                                 cudaStream_t s) {
   const TaylorC t = taylor_c();
+  const fd_status st = coef_attr();
+  if (st) return st;
   const int grid =
-      int(std::max<size_t>(1, std::min<size_t>(size_t(sm_count()) * 3, (ncell + S - 1) / S)));
-  k_mlp_coef<true><<<grid, NTHR, SM_FWD * sizeof(float), s>>>(
+      int(std::max<size_t>(1, std::min<size_t>(size_t(sm_count()) * 4, (ncell + CS - 1) / CS)));
+  k_mlp_coef<true><<<grid, CTHR, SM_COEF * sizeof(float), s>>>(
       net->p, A, ncell, pitch, Nx, float(h / 10.0), float(dt / 1.0), float(f_hz / 10.0), t, coef);
   count_launch();
   cudaError_t e = cudaGetLastError();
@@ -598,9 +692,9 @@ fd_status fd_mlp_create(int32_t device, const float* params, fd_mlp* out) {
   float** bufs[4] = {&net->p, &net->g, &net->m, &net->v};
   for (int i = 0; i < 4 && !e; ++i)
     e = dev_alloc(reinterpret_cast<void**>(bufs[i]), GRAD_BYTES);
-  if (!e) e = cudaMallocHost(reinterpret_cast<void**>(&net->host), GRAD_BYTES);
   if (!e) {
     net->loss = reinterpret_cast<double*>(net->g + NPARAM);
+    net->host.resize(GRAD_BYTES / sizeof(float));
     for (int i = 0; i < 4 && !e; ++i) e = cudaMemsetAsync(*bufs[i], 0, NPARAM * 4, net->stream);
     if (!e && params) e = cudaMemcpyAsync(net->p, params, NPARAM * 4, cudaMemcpyDefault,
                                           net->stream);
@@ -621,7 +715,6 @@ fd_status fd_mlp_destroy(fd_mlp net) {
   if (net->stream) cudaStreamSynchronize(net->stream);
   for (float* p : {net->p, net->g, net->m, net->v})
     if (p) cudaFree(p);
-  if (net->host) cudaFreeHost(net->host);
   net->stage.release();
   net->stage2.release();
   if (net->stream) cudaStreamDestroy(net->stream);
@@ -679,11 +772,11 @@ static fd_status mlp_grad_read(fd_mlp net, double* loss, float* grad) {
   const bool dev = grad && is_device_ptr(grad);
   if (dev) e = cudaMemcpyAsync(grad, net->g, NPARAM * 4, cudaMemcpyDeviceToDevice, net->stream);
   if (!e && (loss || (grad && !dev)))
-    e = cudaMemcpyAsync(net->host, net->g, GRAD_BYTES, cudaMemcpyDeviceToHost, net->stream);
+    e = cudaMemcpyAsync(net->host.data(), net->g, GRAD_BYTES, cudaMemcpyDeviceToHost, net->stream);
   if (!e) e = cudaStreamSynchronize(net->stream);
   if (e) return cuda_fail(e, "gradient read");
-  if (loss) memcpy(loss, net->host + NPARAM, sizeof(double));
-  if (grad && !dev) memcpy(grad, net->host, NPARAM * 4);
+  if (loss) memcpy(loss, net->host.data() + NPARAM, sizeof(double));
+  if (grad && !dev) memcpy(grad, net->host.data(), NPARAM * 4);
   return FD_OK;
 }
 
@@ -788,8 +881,10 @@ fd_status fd_mlp_coefficients(fd_mlp net, int64_t n, const float* features, floa
     cout = static_cast<float*>(net->stage2.p);
   }
   if (e) return cuda_fail(e, "staging");
-  const int grid = int(std::min<int64_t>(sm_count() * 3, (n + S - 1) / S));
-  k_mlp_coef<false><<<grid, NTHR, SM_FWD * sizeof(float), net->stream>>>(
+  const fd_status st = coef_attr();
+  if (st) return st;
+  const int grid = int(std::min<int64_t>(sm_count() * 4, (n + CS - 1) / CS));
+  k_mlp_coef<false><<<grid, CTHR, SM_COEF * sizeof(float), net->stream>>>(
       net->p, fin, size_t(n), 1, 1, 0.f, 0.f, 0.f, taylor_c(), cout);
   count_launch();
   if ((e = cudaGetLastError())) return cuda_fail(e, "inference");
