@@ -31,12 +31,12 @@
 // in step with its neighbours, whose halos it then finds in L2; the rest is
 // cut into G equal contiguous shares of (column, plane) units.
 //
-// What bounds it (ncu, 336^3 at SO 8): latency; the FMA pipes are 42 % busy, the
-// shared-memory pipe 55-65 %, DRAM 63 % of the copy rate at 1.07 x the 48 B per
-// point.  The scalar kernel with separate fields that this replaced executed 523
-// instructions per point at SO 8 and 902 at SO 16, this one 250 and 390:
-// 100 steps of 336^3 at SO 8 80.7 -> 47.1 ms (80.5 Gpts/s), 60 steps of
-// 243 x 181 x 207 at SO 16 31.6 -> 13.4 ms (40.9 Gpts/s).  Equal shares of all
+// What bounds it (ncu, 336^3 at SO 8): shared-memory reads and latency; the
+// shared-memory pipe is 66 % busy, issue 59 %, DRAM 63 % of the copy rate at 1.12 x
+// the 48 B per point.  The scalar kernel with separate fields that this replaced
+// executed 523 instructions per point at SO 8 and 902 at SO 16, this one 280 and
+// 422: 100 steps of 336^3 at SO 8 80.7 -> 46.9 ms (80.9 Gpts/s), 60 steps of
+// 243 x 181 x 207 at SO 16 31.6 -> 12.9 ms (42.3 Gpts/s).  Equal shares of all
 // columns instead of whole waves read 1.67 x the bytes (50.5 ms).
 //
 // Every mbarrier wait is bounded.  A thread whose wait runs out records an
