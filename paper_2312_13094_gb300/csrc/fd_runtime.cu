@@ -580,13 +580,15 @@ void fill_desc(fd_grid g, const RunSpec& rs, ShotDesc* d) {
 // Tile of the plain runs of a grid left on its default tile that the tuner has
 // not seen (runs below kTuneMinSteps): it runs under the wave schedule, whose
 // chunk height balances the resident CTAs for any size.  Of the two tiles of
-// 512 points, 32 x 16 and 64 x 8, the one whose busiest CTA has less to do; on a
-// tie 64 x 8 up to SO 4 (its longer rows) and 32 x 16 (its smaller halo) beyond.
+// 512 points, 32 x 16 and 64 x 8, the one whose busiest CTA has less to do.  Where
+// that hardly differs, 64 x 8 (longer rows) up to SO 6 and on larger grids at SO 8,
+// 32 x 16 (less halo) beyond.
 // Measured (us a step, 32 x 16 / 64 x 8 / the equal shares on default_shape
 // that such runs had before): 251 x 197 x 163 SO 8 31.3 / 32.0 / 36.4;
 // 200 x 240 x 280 SO 8 47.7 / 54.8 / 49.8; 190^3 SO 12 36.9 / 37.2 / 57.6;
-// 300^3 SO 4 95.0 / 86.6 / -; 440 x 340 x 370 SO 16 304 / 249 / -.  The predicted
-// loads of the last are 282 and 205 planes.
+// 226 x 486 x 143 SO 6 55.8 / 51.9 / 52.8; 349 x 341 x 288 SO 2 106 / 102 / 110;
+// gradient steps of 296^3 SO 8 106 / 103 / 104; 440 x 340 x 370 SO 16 304 / 249 / -,
+// with predicted loads of 282 and 205 planes.
 static TileShape wave_tile(fd_grid g) {
   if (g->wave_shape.tx == 0) {
     const TileShape shapes[2] = {{8, 16, 1, 0}, {16, 8, 2, 0}};
@@ -596,7 +598,8 @@ static TileShape wave_tile(fd_grid g) {
       const int tiles = ((g->Nx + bx - 1) / bx) * ((g->Ny + by - 1) / by);
       load[i] = wave_load({{0, tiles, g->Nz}}, sweep_ctas(g->R, shapes[i], kModeForward), g->R);
     }
-    g->wave_shape = shapes[load[1] < load[0] || (load[1] == load[0] && g->R <= 2) ? 1 : 0];
+    const bool rows = g->R <= 3 || (g->R == 4 && (long long)g->Nx * g->Ny * g->Nz > 16000000);
+    g->wave_shape = shapes[rows ? load[1] <= load[0] + load[0] / 50 : load[1] < load[0]];
   }
   return g->wave_shape;
 }
@@ -755,6 +758,14 @@ fd_status autotune_grid(fd_grid g) {
         pick = {t, g->tuned_waves};
       }
     }
+    // Pairs within a percent or two of the fastest are ranked by chance, and the
+    // adjoint's steps, which take the pick too, are not: of those, waves on
+    // wave_tile (296^3 SO 8, us a forward step / mean of a gradient's three: 64 x 8
+    // waves 79.6 / 103.2, shares 80.9 / 103.9, 32 x 16 waves 80.5 / 106.3)
+    const TileShape w = wave_tile(g);
+    for (int i = 0; i < kNumShapes; ++i)
+      if (kShapes[i].tx == w.tx && kShapes[i].ty == w.ty && best_of[2 * i + 1] <= 1.02f * best)
+        pick = {kShapes[i], true};
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
     g->profiling = prof;
