@@ -24,6 +24,7 @@ namespace {
 
 struct BatchWorkspace {
   DevBuf desc;  // ShotDesc[nshots] followed by the unit prefix [nshots + 1]
+  cudaEvent_t staged = nullptr;  // behind one grid's uploads, on its own stream
   bool graph_valid = false;
   cudaGraphExec_t gexec = nullptr;
   std::vector<char> key;
@@ -94,10 +95,23 @@ struct Prepared {
   long long spin_limit = 0;
 };
 
+// Lets stream s, on which the batch runs, wait for all that grid g's own stream
+// holds: the tables and wavelet just staged there, and work queued before them
+// (a wavelet that the caller's kernels still write, say).
+fd_status join_stream(BatchWorkspace& ws, fd_grid g, cudaStream_t s) {
+  if (g->stream == s) return FD_OK;
+  cudaError_t e = cudaSuccess;
+  if (!ws.staged) e = cudaEventCreateWithFlags(&ws.staged, cudaEventDisableTiming);
+  if (!e) e = cudaEventRecord(ws.staged, g->stream);
+  if (!e) e = cudaStreamWaitEvent(s, ws.staged, 0);
+  return e ? cuda_fail(e, "batch stream order") : FD_OK;
+}
+
 // Puts every shot on tile shape t and builds the descriptors and the unit
-// prefix of the batch.
-fd_status prepare(int nshots, const fd_shot* shots, const TileShape& t, bool waves,
-                  Prepared& P) {
+// prefix of the batch.  Each grid's tables and wavelet go up on its own stream,
+// which stream s of the batch then waits for.
+fd_status prepare(BatchWorkspace& ws, int nshots, const fd_shot* shots, const TileShape& t,
+                  bool waves, cudaStream_t s, Prepared& P) {
   const int R = shots[0].grid->R;
   P.nshots = nshots;
   P.drec.assign(nshots, nullptr);
@@ -125,6 +139,7 @@ fd_status prepare(int nshots, const fd_shot* shots, const TileShape& t, bool wav
     if ((st = stage_out(g, g->stage_rec, nrec ? shots[i].rec_out : nullptr,
                         size_t(g->d.nt) * nrec, &drec)))
       return st;
+    if ((st = join_stream(ws, g, s))) return st;
     P.drec[i] = drec;
     RunSpec rs;
     memset(&rs, 0, sizeof(rs));
@@ -232,7 +247,7 @@ fd_status autotune(BatchWorkspace& ws, int nshots, const fd_shot* shots, int R, 
     TileShape t = kShapes[c / 2];
     const bool waves = (c & 1) != 0;
     Prepared P;
-    st = prepare(nshots, shots, t, waves, P);
+    st = prepare(ws, nshots, shots, t, waves, s, P);
     if (!st) st = upload_prepared(ws, P, s);
     if (!st) st = zero_state(nshots, shots, s);
     if (!st) st = issue_steps(ws, P, R, t, 1, s);  // warm-up
@@ -305,7 +320,7 @@ extern "C" fd_status fd_batch_forward(int32_t nshots, const fd_shot* shots, int3
   const TileShape t = pick.t;
 
   Prepared P;
-  if ((st = prepare(nshots, shots, t, pick.waves, P))) return st;
+  if ((st = prepare(ws, nshots, shots, t, pick.waves, s, P))) return st;
   if ((st = upload_prepared(ws, P, s))) return st;
   if ((st = zero_state(nshots, shots, s))) return st;
 

@@ -134,6 +134,8 @@ extern "C" fd_status fd_forward_noalloc(const fd_grid_desc* d, const float* mode
   // set_model clears both wavefields; fd_forward clears them again
   if (!st) st = fd_set_model(&g, model, kind);
   if (!st) st = fd_forward(&g, src, wavelet, rec, rec_out, nullptr);
+  // an error may have left copies of the images that the stack grid holds under way
+  if (!g.held.empty()) cudaStreamSynchronize(g.stream);
   // the stack grid owns nothing: detach every pointer before it goes away
   for (int i = 0; i < 5; ++i) {
     bufs[i]->p = nullptr;

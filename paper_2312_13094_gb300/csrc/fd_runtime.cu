@@ -435,16 +435,24 @@ fd_status build_receivers(fd_grid g, const fd_points* pts, std::vector<int32_t>&
   return build_receivers_tiles(g, pts, 4 * g->shape.tx, g->shape.ty, start, out);
 }
 
+fd_status copy_in(fd_grid g, void* dst, const void* src, size_t bytes, const char* what) {
+  constexpr size_t kMostHeld = 4096;  // reached only where run after run ends in an error
+  cudaError_t e = cudaSuccess;
+  if (g->held.size() >= kMostHeld && !(e = cudaStreamSynchronize(g->stream))) g->held.clear();
+  if (!e) {
+    const char* p = static_cast<const char*>(src);
+    g->held.emplace_back(p, p + bytes);
+    e = cudaMemcpyAsync(dst, g->held.back().data(), bytes, cudaMemcpyHostToDevice, g->stream);
+  }
+  return e ? cuda_fail(e, what) : FD_OK;
+}
+
 template <class T>
 fd_status upload(fd_grid g, DevBuf& buf, const std::vector<T>& v) {
   cudaError_t e = buf.ensure(std::max<size_t>(v.size() * sizeof(T), 16));
   if (e) return cuda_fail(e, "table allocation");
-  if (!v.empty()) {
-    e = cudaMemcpyAsync(buf.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice,
-                        g->stream);
-    if (e) return cuda_fail(e, "table upload");
-  }
-  return FD_OK;
+  if (v.empty()) return FD_OK;
+  return copy_in(g, buf.p, v.data(), v.size() * sizeof(T), "table upload");
 }
 template fd_status upload<int32_t>(fd_grid, DevBuf&, const std::vector<int32_t>&);
 template fd_status upload<InjEntry>(fd_grid, DevBuf&, const std::vector<InjEntry>&);
@@ -465,8 +473,6 @@ fd_status upload_tables(fd_grid g, const fd_points* src, double src_scale,
   if ((st = upload(g, t.recs, re))) return st;
   t.n_inj = int(ie.size());
   t.n_rec = int(re.size());
-  // (an asynchronous copy from pageable memory has read it when it returns, so
-  // the vectors may go away)
   return FD_OK;
 }
 
@@ -831,8 +837,7 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
   e = g->desc.ensure(2 * sizeof(host));
   if (e) return cuda_fail(e, "descriptor allocation");
   char* dslot = static_cast<char*>(g->desc.p) + slot * sizeof(host);
-  e = cudaMemcpyAsync(dslot, &host, sizeof(host), cudaMemcpyHostToDevice, g->stream);
-  if (e) return cuda_fail(e, "descriptor upload");
+  if (fd_status st = copy_in(g, dslot, &host, sizeof(host), "descriptor upload")) return st;
   const ShotDesc* dshot = reinterpret_cast<const ShotDesc*>(dslot);
   const long long* dprefix = reinterpret_cast<const long long*>(dslot + sizeof(ShotDesc));
 
@@ -932,6 +937,7 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
 fd_status check_device_error(fd_grid g) {
   cudaError_t e = cudaStreamSynchronize(g->stream);
   if (e) return cuda_fail(e, "stream synchronize");
+  g->held.clear();
   int h = 0;
   e = cudaMemcpy(&h, g->d_err, sizeof(int), cudaMemcpyDeviceToHost);
   if (e) return cuda_fail(e, "error word read");
@@ -958,6 +964,7 @@ fd_status check_run(fd_grid g, const float* rec, size_t n) {
   if (!e) e = cudaMemcpyAsync(h, g->d_err, sizeof(h), cudaMemcpyDeviceToHost, g->stream);
   if (!e) e = cudaStreamSynchronize(g->stream);
   if (e) return cuda_fail(e, "run check");
+  g->held.clear();
   if (h[0]) {
     cudaMemset(g->d_err, 0, sizeof(int));
     return fail(FD_ERR_TIMEOUT, "a device-side wait ran out (error word %d)", h[0]);

@@ -108,6 +108,8 @@ struct fd_grid_s {
   fd::DevBuf stage_val, stage_rec, stage_aux, recbuf;
   fd::DevBuf ckpt, ebuf, gpad, resid;
   fd::DevBuf desc;  // sweep descriptors (forward and adjoint slots)
+  // host images of tables and descriptors whose copies may be under way (copy_in)
+  std::vector<std::vector<char>> held;
   int32_t* d_err = nullptr;  // [0] wait-timeout word, [1] finite count, [4..6] scratch
   long long spin_limit = 0;
   int debug_skip_plane = -1;
@@ -190,6 +192,11 @@ fd_status build_injection_tiles(fd_grid g, const fd_points* pts, double scale, i
                                 std::vector<InjEntry>& out);
 fd_status build_receivers_tiles(fd_grid g, const fd_points* pts, int bx, int by,
                                 std::vector<int32_t>& start, std::vector<RecEntry>& out);
+// Copies host memory that need not outlive the call to the device, on the grid's
+// stream.  An asynchronous copy from pageable memory is only sometimes a
+// synchronous one, so the grid holds an image of the bytes until the run has been
+// waited for (check_run, check_device_error).
+fd_status copy_in(fd_grid g, void* dst, const void* src, size_t bytes, const char* what);
 // Host vector to a device buffer (grown as needed) on the grid's stream.
 template <class T>
 fd_status upload(fd_grid g, DevBuf& buf, const std::vector<T>& v);

@@ -150,8 +150,8 @@ fd_status tblock_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
   a.A = g->A;
   a.err = g->d_err;
   cudaError_t e = t->desc.ensure(sizeof(TbDesc));
-  if (!e) e = cudaMemcpyAsync(t->desc.p, &host, sizeof(host), cudaMemcpyHostToDevice, g->stream);
   if (e) return cuda_fail(e, "two-step descriptor");
+  if ((st = copy_in(g, t->desc.p, &host, sizeof(host), "two-step descriptor"))) return st;
 
   TbLaunch L;
   memset(&L, 0, sizeof(L));
