@@ -712,15 +712,18 @@ static_assert(NPARAM * 4 % sizeof(double) == 0, "loss alignment");
 struct fd_mlp_s {
   int device = 0;
   cudaStream_t stream = nullptr;
+  void* mem = nullptr;  // one allocation for all of the following
   float* p = nullptr;   // params
   float* g = nullptr;   // gradient
   float* m = nullptr;   // Adam first moment
   float* v = nullptr;   // Adam second moment
-  double* loss = nullptr;  // behind the gradient in its allocation
+  double* loss = nullptr;  // behind the gradient
+  double* lpart = nullptr;  // losses and gradient sums of the training kernel's blocks,
+  float* part = nullptr;    // for as many blocks as it launches at most
+  int most_blocks = 0;
   std::vector<float> host;  // image of gradient and loss
   int t = 0;               // Adam step count
   DevBuf stage, stage2;
-  DevBuf part;             // gradient sums and losses of the training kernel's blocks
 };
 
 namespace fd {
@@ -756,9 +759,16 @@ fd_status fd_mlp_create(int32_t device, const float* params, fd_mlp* out) {
   fd_status st = FD_OK;
   e = cudaStreamCreateWithFlags(&net->stream, cudaStreamDefault);  // see fd_create_grid
   float** bufs[4] = {&net->p, &net->g, &net->m, &net->v};
-  for (int i = 0; i < 4 && !e; ++i)
-    e = dev_alloc(reinterpret_cast<void**>(bufs[i]), GRAD_BYTES);
+  constexpr size_t kField = (GRAD_BYTES + 255) / 256 * 256;
+  net->most_blocks = 2 * std::max(1, sm_count());  // two per SM
+  if (!e)
+    e = dev_alloc(&net->mem, 4 * kField + size_t(net->most_blocks) *
+                                              (NPARAM * 4 + NWARP * sizeof(double)));
   if (!e) {
+    char* q = static_cast<char*>(net->mem);
+    for (int i = 0; i < 4; ++i, q += kField) *bufs[i] = reinterpret_cast<float*>(q);
+    net->lpart = reinterpret_cast<double*>(q);
+    net->part = reinterpret_cast<float*>(net->lpart + size_t(net->most_blocks) * NWARP);
     net->loss = reinterpret_cast<double*>(net->g + NPARAM);
     net->host.resize(GRAD_BYTES / sizeof(float));
     for (int i = 0; i < 4 && !e; ++i) e = cudaMemsetAsync(*bufs[i], 0, NPARAM * 4, net->stream);
@@ -779,11 +789,9 @@ fd_status fd_mlp_destroy(fd_mlp net) {
   if (!net) return FD_OK;
   cudaSetDevice(net->device);
   if (net->stream) cudaStreamSynchronize(net->stream);
-  for (float* p : {net->p, net->g, net->m, net->v})
-    if (p) cudaFree(p);
+  if (net->mem) cudaFree(net->mem);
   net->stage.release();
   net->stage2.release();
-  net->part.release();
   if (net->stream) cudaStreamDestroy(net->stream);
   delete net;
   return FD_OK;
@@ -825,22 +833,17 @@ static fd_status mlp_grad_device(fd_mlp net, int64_t n, const float* dsamples) {
     if (e) return cuda_fail(e, "kernel attribute");
     attr = true;
   }
-  // two blocks per SM; a small batch is spread one warp's samples per block
-  const int most = 2 * sm_count();
-  const int blocks = int(std::min<int64_t>(most, (n + NSUB - 1) / NSUB));
-  if ((e = net->part.ensure(size_t(most) * (NPARAM * 4 + NWARP * sizeof(double)))))
-    return cuda_fail(e, "gradient workspace");
-  double* lpart = static_cast<double*>(net->part.p);
-  float* part = reinterpret_cast<float*>(lpart + size_t(most) * NWARP);
+  // a small batch is spread one warp's samples per block
+  const int blocks = int(std::min<int64_t>(net->most_blocks, (n + NSUB - 1) / NSUB));
   k_mlp_grad<<<blocks, NTHR, SM_GRAD * sizeof(float), net->stream>>>(
-      net->p, dsamples, int(n), float(1.0 / double(n)), taylor_c(), part, lpart);
+      net->p, dsamples, int(n), float(1.0 / double(n)), taylor_c(), net->part, net->lpart);
   count_launch(2);
   e = cudaGetLastError();
   // (may start while the last blocks of the training kernel run: it waits itself)
   if (!e)
     e = launch_step(k_mlp_sum, dim3((NPARAM + 4 * SW - 1) / (4 * SW) + 1), SW * SR, 0, true,
-                    net->stream, static_cast<const float*>(part),
-                    static_cast<const double*>(lpart), blocks, net->g, net->loss);
+                    net->stream, static_cast<const float*>(net->part),
+                    static_cast<const double*>(net->lpart), blocks, net->g, net->loss);
   if (e) return cuda_fail(e, "training kernel");
   return FD_OK;
 }
