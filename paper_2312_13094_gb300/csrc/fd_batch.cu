@@ -223,6 +223,7 @@ fd_status issue_steps(BatchWorkspace& ws, const Prepared& P, int R, const TileSh
     ov.rec_row = step;
     ov.spin_limit = P.spin_limit;
     ov.debug_skip_plane = -1;
+    ov.fresh = step == 0 ? P.nshots : 0;
     for (int j = 0; j < kMaxR + 2; ++j) ov.c[j] = P.c[j];
     if (P.waves) {
       const char* base = static_cast<const char*>(ws.desc.p);

@@ -564,6 +564,7 @@ fd_status cart_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
       ov.rec_row = t;
       ov.spin_limit = g->spin_limit;
       ov.debug_skip_plane = -1;
+      ov.fresh = t == 0 ? nbox : 0;
       ov.item_start = item_start;
       ov.items = items;
       launch_weights(g->c, R, ov.c);

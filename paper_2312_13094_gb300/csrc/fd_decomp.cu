@@ -343,6 +343,7 @@ fd_status decomp_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
       ov.rec_row = t;
       ov.spin_limit = g->spin_limit;
       ov.debug_skip_plane = -1;
+      ov.fresh = t == 0 ? 1 : 0;
       launch_weights(g->c, R, ov.c);
       const ShotDesc* sd = reinterpret_cast<const ShotDesc*>(base + i * kBlock);
       const long long* pf = reinterpret_cast<const long long*>(base + i * kBlock + sizeof(ShotDesc));

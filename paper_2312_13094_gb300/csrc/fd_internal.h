@@ -111,6 +111,8 @@ struct StepOverride {
                              // centre weight's lo part
   const int32_t* item_start; // scheduled sweep: CTA c runs items [item_start[c],
   const WorkItem* items;     // item_start[c+1]); nullptr: equal contiguous shares
+  int fresh;                 // first launch since the tensor maps in device memory may
+                             // have changed: grids whose maps it acquires (else 0)
 };
 
 // Two-step (temporally blocked) pass, fd_tblock.cuh: what does not change
@@ -154,6 +156,7 @@ struct TbLaunch {
   float c[kMaxR + 2];  // as StepOverride::c
   const int32_t* item_start;
   const WorkItem* items;
+  int fresh;           // first pass of a run: acquire the tensor maps
 };
 
 // The weights of a uniform-stencil launch from the FP64 weights c[0..R]

@@ -108,6 +108,7 @@ struct fd_grid_s {
   fd::DevBuf stage_val, stage_rec, stage_aux, recbuf;
   fd::DevBuf ckpt, ebuf, gpad, resid;
   fd::DevBuf desc;  // sweep descriptors (forward and adjoint slots)
+  std::vector<char> sent_maps[2];  // tensor maps that each slot of desc holds
   // host images of tables and descriptors whose copies may be under way (copy_in)
   std::vector<std::vector<char>> held;
   int32_t* d_err = nullptr;  // [0] wait-timeout word, [1] finite count, [4..6] scratch

@@ -172,6 +172,7 @@ fd_status tblock_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
     L.out2 = other + 1;
     L.inj_row = n0 + 2 * p;
     L.rec_row = 2 * p;
+    L.fresh = p == 0;
     count_launch();
     e = R == 2 ? launch_tblock_r<2>(dd, L, t->sched_ctas, g->stream)
                : launch_tblock_r<4>(dd, L, t->sched_ctas, g->stream);
