@@ -8,32 +8,59 @@ namespace fd {
 
 namespace {
 
-__global__ void k_model_stats(const float* __restrict__ data, size_t n, int kind,
-                              unsigned int* vmin_bits, unsigned int* vmax_bits,
-                              int* bad) {
-  float lo = INFINITY, hi = 0.0f;
-  int nbad = 0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const float x = data[i];
+// Smallest and largest velocity of a model and its count of bad values.  Bound by
+// memory: four loads of a thread are in flight, on up to eight blocks per SM.  The
+// maxima of a block go to the words in one atomic each (one per thread queued 2.6e5
+// of them on each word; one per warp and two blocks per SM left too few loads in
+// flight for large models).  fd_set_model of 64^3 / 256^3 / 512^3 cells, us: with one
+// atomic per thread and 1024 blocks 63 / 328 / 1772, with one per warp and two blocks
+// per SM 54 / 387 / 2316, now 52 / 303 / 1634.
+constexpr int kStatThreads = 256, kStatLoads = 4;
+__global__ void __launch_bounds__(kStatThreads)
+    k_model_stats(const float* __restrict__ data, size_t n, int kind, unsigned int* vmin_bits,
+                  unsigned int* vmax_bits, int* bad) {
+  // positive floats order like their bit patterns
+  unsigned lo = 0x7f800000u, hi = 0u, nbad = 0u;
+  auto take = [&](float x) {
     if (!(x > 0.0f) || !isfinite(x)) {
       ++nbad;
-      continue;
+      return;
     }
-    const float v = kind == 0 ? x : 1.0f / sqrtf(x);
-    lo = fminf(lo, v);
-    hi = fmaxf(hi, v);
+    const unsigned v = __float_as_uint(kind == 0 ? x : 1.0f / sqrtf(x));
+    lo = min(lo, v);
+    hi = max(hi, v);
+  };
+  const size_t step = (size_t)gridDim.x * kStatThreads;
+  size_t i = blockIdx.x * (size_t)kStatThreads + threadIdx.x;
+  for (; i + (kStatLoads - 1) * step < n; i += kStatLoads * step) {
+    float x[kStatLoads];
+#pragma unroll
+    for (int k = 0; k < kStatLoads; ++k) x[k] = data[i + k * step];
+#pragma unroll
+    for (int k = 0; k < kStatLoads; ++k) take(x[k]);
   }
-  // positive floats order like their bit patterns; one atomic per warp (one
-  // per thread queued 2.6e5 of them on each word)
-  const unsigned lo_bits = __reduce_min_sync(0xffffffffu, __float_as_uint(lo));
-  const unsigned hi_bits = __reduce_max_sync(0xffffffffu, __float_as_uint(hi));
+  for (; i < n; i += step) take(data[i]);
+  __shared__ unsigned s_lo[kStatThreads / 32], s_hi[kStatThreads / 32], s_bad[kStatThreads / 32];
+  __syncwarp();
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
   nbad = __reduce_add_sync(0xffffffffu, nbad);
-  if ((threadIdx.x & 31) != 0) return;
-  if (nbad) atomicAdd(bad, nbad);
-  if (hi_bits) {
-    atomicMin(vmin_bits, lo_bits);
-    atomicMax(vmax_bits, hi_bits);
+  if ((threadIdx.x & 31) == 0) {
+    s_lo[threadIdx.x >> 5] = lo;
+    s_hi[threadIdx.x >> 5] = hi;
+    s_bad[threadIdx.x >> 5] = nbad;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < kStatThreads / 32; ++w) {
+    lo = min(lo, s_lo[w]);
+    hi = max(hi, s_hi[w]);
+    nbad += s_bad[w];
+  }
+  if (nbad) atomicAdd(bad, static_cast<int>(nbad));
+  if (hi) {
+    atomicMin(vmin_bits, lo);
+    atomicMax(vmax_bits, hi);
   }
 }
 
@@ -142,12 +169,18 @@ cudaError_t pad_coefficients(const float* phys, int R, int nx, int ny, int nz, i
 cudaError_t model_stats(const float* data, size_t n, int kind, float* vmin,
                         float* vmax, int* nbad, unsigned int* scratch,
                         cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   // scratch: [vmin_bits, vmax_bits, bad]
   unsigned int init[3] = {0x7f800000u, 0u, 0u};
-  cudaError_t e = cudaMemcpyAsync(scratch, init, sizeof(init), cudaMemcpyHostToDevice, s);
+  e = cudaMemcpyAsync(scratch, init, sizeof(init), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
-  k_model_stats<<<304, 256, 0, s>>>(data, n, kind, scratch, scratch + 1,
-                                     reinterpret_cast<int*>(scratch + 2));
+  const size_t want = (n + kStatThreads * kStatLoads - 1) / (kStatThreads * kStatLoads);
+  const int blocks = int(want < 1 ? 1 : (want < size_t(8) * sms ? want : size_t(8) * sms));
+  k_model_stats<<<blocks, kStatThreads, 0, s>>>(data, n, kind, scratch, scratch + 1,
+                                                reinterpret_cast<int*>(scratch + 2));
   count_launch();
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   unsigned int out[3];
