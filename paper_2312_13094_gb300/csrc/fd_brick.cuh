@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(BrickCfg<R, MODE>::NT, BrickCfg<R, MODE>::CTAS
   const int cur = ov.cur;
   pdl_trigger();
   if (ov.fresh) {
-    acquire_maps<MODE>(shot, 1);
+    acquire_maps(shot, 1);
     __syncwarp();  // before the prefetch; before the copies, the barrier below
   }
   if (tid < 3)  // the tensor maps, fetched while the step ahead still runs

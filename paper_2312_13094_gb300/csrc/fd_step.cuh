@@ -186,13 +186,12 @@ __device__ __forceinline__ void acquire_map(const CUtensorMap* map) {
 // 5 us one of 149 x 128 x 103 (12 us).  Passing the maps as kernel parameters, which
 // needs no fence, cost that gradient 1 us a step, as each launch then brings maps
 // at an address that no SM has seen.
-template <int MODE>
 __device__ __forceinline__ void acquire_maps(const ShotDesc* shots, int nshots) {
   static_assert(offsetof(ShotDesc, tile) == 2 * sizeof(CUtensorMap) &&
                     offsetof(ShotDesc, A) == 4 * sizeof(CUtensorMap) &&
                     offsetof(ShotDesc, C) == 5 * sizeof(CUtensorMap),
                 "halo[2], tile[2], A, C");
-  constexpr int kMaps = MODE == kModePerCell ? 6 : 5;
+  constexpr int kMaps = 6;  // C too: a later run with per-cell weights may find them unchanged
   for (int i = threadIdx.x; i < kMaps * nshots; i += blockDim.x)
     acquire_map(shots[i / kMaps].halo + i % kMaps);
 }
@@ -895,7 +894,7 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
   const long long hi = total * (blockIdx.x + 1) / gridDim.x;
   const int cur = ov.cur;
   pdl_trigger();
-  if (ov.fresh) acquire_maps<MODE>(shots, ov.fresh);
+  if (ov.fresh) acquire_maps(shots, ov.fresh);
   pdl_wait();
   int s = 0;
   for (long long pos = lo; pos < hi;) {
@@ -938,7 +937,7 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
   const int cur = ov.cur;
   const int i1 = ov.item_start[blockIdx.x + 1];
   pdl_trigger();
-  if (ov.fresh) acquire_maps<MODE>(shots, ov.fresh);
+  if (ov.fresh) acquire_maps(shots, ov.fresh);
   pdl_wait();
   for (int i = ov.item_start[blockIdx.x]; i < i1; ++i) {
     const WorkItem w = ov.items[i];
