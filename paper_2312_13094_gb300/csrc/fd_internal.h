@@ -175,6 +175,13 @@ inline void launch_weights(const double* c, int R, float* out) {
   out[kMaxR + 1] = static_cast<float>(t - static_cast<double>(out[0]));
 }
 
+// Whether a kernel on `device` may address memory that cudaPointerGetAttributes
+// describes so: its own, or managed memory.  Memory of another device is left to
+// copies, which need no peer access.
+inline bool kernel_can_address(cudaMemoryType type, int owner, int device) {
+  return type == cudaMemoryTypeManaged || (type == cudaMemoryTypeDevice && owner == device);
+}
+
 struct TileShape {
   int tx, ty, pf;   // threads in x (4 points each), rows, prefetch depth
   int ctas;         // persistent CTAs per sweep (0: resident CTAs per SM x SMs)

@@ -107,6 +107,16 @@ bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+bool is_local_ptr(const void* p, int device) {
+  if (!p) return false;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return kernel_can_address(at.type, at.device, device);
+}
+
 // --------------------------------------------------------------------------
 // tensor maps
 // --------------------------------------------------------------------------

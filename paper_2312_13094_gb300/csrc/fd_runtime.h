@@ -148,6 +148,7 @@ cudaError_t dev_alloc(void** p, size_t bytes);
 long long alloc_count();         // device allocations made through dev_alloc so far
 long long default_spin_limit();  // FD_SPIN_LIMIT, else ~0.1 s of clock cycles
 bool is_device_ptr(const void* p);
+bool is_local_ptr(const void* p, int device);  // a kernel on `device` may address it
 fd_status make_map(CUtensorMap* m, const float* base, int Nx, int Ny, int Nz, int pitch, int bx,
                    int by);
 int radius_halo_x(int R);

@@ -76,7 +76,7 @@ struct fd_tti_s {
 
 namespace {
 
-constexpr size_t kStageBytes = size_t(32) << 20;  // staging of host states
+constexpr size_t kStageBytes = size_t(32) << 20;  // staging of states not on the device
 
 struct TtiInj {
   long long off;
@@ -348,11 +348,11 @@ fd_status tables(fd_tti t, const fd_points* src, const fd_points* rec) {
 }
 
 // One field of a state (f = 0: p, 1: q) between its pairs and a dense padded
-// array of the caller, device memory directly, host memory through a staging
-// buffer in pieces of whole rows.
+// array of the caller: memory of the grid's own device directly, host memory and
+// that of other devices through a staging buffer in pieces of whole rows.
 fd_status copy_state(fd_tti t, float2* dev, int f, void* user, bool to_user) {
   const size_t rows = size_t(t->Ny) * t->Nz;
-  const bool on_device = is_device_ptr(user);
+  const bool on_device = is_local_ptr(user, t->d.device);
   const size_t row_bytes = size_t(t->Nx) * 4;
   const size_t most = 65535;  // rows of one launch
   const size_t piece =
@@ -366,7 +366,7 @@ fd_status copy_state(fd_tti t, float2* dev, int f, void* user, bool to_user) {
     char* u = static_cast<char*>(user) + r * row_bytes;
     float* dense = static_cast<float*>(on_device ? static_cast<void*>(u) : t->stage_in.p);
     if (!on_device && !to_user) {
-      e = cudaMemcpyAsync(dense, u, n * row_bytes, cudaMemcpyHostToDevice, t->stream);
+      e = cudaMemcpyAsync(dense, u, n * row_bytes, cudaMemcpyDefault, t->stream);
       if (e) return cuda_fail(e, "wavefield copy");
     }
     k_tti_field<<<dim3((t->Nx + 127) / 128, unsigned(n)), 128, 0, t->stream>>>(
@@ -374,7 +374,7 @@ fd_status copy_state(fd_tti t, float2* dev, int f, void* user, bool to_user) {
     count_launch();
     if ((e = cudaGetLastError())) return cuda_fail(e, "wavefield copy");
     if (!on_device && to_user) {
-      e = cudaMemcpyAsync(u, dense, n * row_bytes, cudaMemcpyDeviceToHost, t->stream);
+      e = cudaMemcpyAsync(u, dense, n * row_bytes, cudaMemcpyDefault, t->stream);
       if (e) return cuda_fail(e, "wavefield copy");
     }
   }
