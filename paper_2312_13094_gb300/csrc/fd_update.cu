@@ -13,10 +13,10 @@
 #include <string.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "fd_aux.h"
 #include "fd_runtime.h"
+#include "fd_slots.h"
 
 namespace fd {
 namespace {
@@ -88,19 +88,16 @@ extern "C" fd_status fd_descent_step(int64_t n, float* m, const float* grad, dou
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   unsigned int* scratch = nullptr;
   cudaError_t e = cudaSuccess;
-  int slot = 0;
-  while (slot < kSlots && g_taken[slot].exchange(true)) ++slot;
-  if (slot < kSlots) {
+  auto wait = [s] { cudaStreamSynchronize(s); };
+  ScratchSlot<kSlots, decltype(wait)> slot(g_taken, wait);
+  if (slot.index() < kSlots) {
     void* base = nullptr;
     e = cudaGetSymbolAddress(&base, g_scratch);  // of the current device
-    scratch = static_cast<unsigned int*>(base) + 4 * slot;
+    scratch = static_cast<unsigned int*>(base) + 4 * slot.index();
   } else {
     e = dev_alloc(reinterpret_cast<void**>(&scratch), 4 * sizeof(unsigned int));
   }
-  if (e) {
-    if (slot < kSlots) g_taken[slot] = false;
-    return cuda_fail(e, "update scratch allocation");
-  }
+  if (e) return cuda_fail(e, "update scratch allocation");
   unsigned int h[4] = {0, 0, 0, 0};
   const int nb = blocks_for(size_t(n));
   e = cudaMemsetAsync(scratch, 0, sizeof(h), s);
@@ -111,6 +108,7 @@ extern "C" fd_status fd_descent_step(int64_t n, float* m, const float* grad, dou
   }
   if (!e) e = cudaMemcpyAsync(h, scratch, sizeof(h), cudaMemcpyDeviceToHost, s);
   if (!e) e = cudaStreamSynchronize(s);
+  if (!e) slot.idle();  // the words have been read, and k_descent takes none
   fd_status st = FD_OK;
   if (e) {
     st = cuda_fail(e, "gradient maxima");
@@ -131,10 +129,6 @@ extern "C" fd_status fd_descent_step(int64_t n, float* m, const float* grad, dou
     }
     if (!st && alpha_out) *alpha_out = alpha;
   }
-  // (the stream has been waited for: nothing reads the words any more)
-  if (slot < kSlots)
-    g_taken[slot] = false;
-  else
-    cudaFree(scratch);
+  if (slot.index() >= kSlots) cudaFree(scratch);
   return st;
 }
