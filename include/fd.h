@@ -95,7 +95,8 @@ typedef struct {
 typedef struct {
   int32_t nx_pad, ny_pad, nz_pad; /* padded (physical + 2 nbl) extents */
   int32_t pitch;                  /* floats between rows of device arrays */
-  int32_t tile_x, tile_y, ctas;   /* stencil tile and persistent CTAs per sweep */
+  int32_t tile_x, tile_y, ctas;   /* stencil tile and CTAs per step: persistent ones,
+                                     or one per brick of a grid that runs on bricks */
   double v_max;                   /* from the model, km/s */
   double cfl_limit;               /* largest stable v_max dt / h */
   int64_t launches;               /* library kernels launched so far */

@@ -18,9 +18,9 @@ cudaError_t model_stats(const float* data, size_t n, int kind, float* vmin,
 cudaError_t model_to_A(const float* data, int kind, int nx, int ny, int nz, int nbl,
                        int Nx, int Ny, int Nz, int pitch, double dt2_h2, float* A,
                        cudaStream_t s);
-// Number of NaN/Inf values in x (synchronises `s`).
-// The count into *dcnt (device), without waiting for it.
+// Number of NaN/Inf values in x into *dcnt (device), without waiting for it.
 cudaError_t count_nonfinite_async(const float* x, size_t n, int* dcnt, cudaStream_t s);
+// The same, read into *hcnt (synchronises `s`).
 cudaError_t count_nonfinite(const float* x, size_t n, int* dcnt, int* hcnt,
                             cudaStream_t s);
 // r = rec - obs and *dloss = sum r^2 / 2 (double, on the device).

@@ -696,10 +696,10 @@ static cudaError_t launch_brick(int R, int mode, const ShotDesc* shot, const Ste
   return cudaErrorInvalidValue;
 }
 
-fd_status use_shape(fd_grid g, bool plain_forward) {
+fd_status use_shape(fd_grid g, bool own_steps) {
   const TileShape want =
-      plain_forward && brick_grid(g) ? kBrickTile
-      : !plain_forward || g->sched_mode != FD_SCHED_AUTO
+      own_steps && brick_grid(g) ? kBrickTile
+      : !own_steps || g->sched_mode != FD_SCHED_AUTO
           ? g->base_shape
           : (g->tuned ? g->tuned_shape : (g->auto_tile ? wave_tile(g) : g->base_shape));
   if (want.tx == 0) return FD_OK;  // a grid without a base tile keeps its own
@@ -825,14 +825,15 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
                 : lockstep_ctas(g->R, g->shape, mode, (long long)g->tiles_x * g->tiles_y, g->Nz);
   StepOverride sched_ov;
   memset(&sched_ov, 0, sizeof(sched_ov));
+  const bool forward_run = mode == kModeForward || mode == kModeTable || mode == kModePerCell;
   if (brick) {
-    if (mode == kModeForward || mode == kModeTable) g->last_sched = FD_SCHED_SHARES;
+    if (forward_run) g->last_sched = FD_SCHED_SHARES;
   } else {
     fd_status st = FD_OK;
     const int Gs = grid_schedule(g, mode, &sched_ov, &st);
     if (st) return st;
     if (Gs > 0) G = Gs;
-    if (mode == kModeForward || mode == kModeTable)
+    if (forward_run)
       g->last_sched = Gs > 0 ? FD_SCHED_WAVES : FD_SCHED_SHARES;
   }
   // descriptor + unit prefix, refreshed before every run (stream ordered),
@@ -1338,7 +1339,10 @@ fd_status fd_get_info(fd_grid g, fd_grid_info* info) {
   info->pitch = g->pitch;
   info->tile_x = 4 * g->shape.tx;
   info->tile_y = g->shape.ty;
-  info->ctas = sweep_ctas(g->R, g->shape, forward_mode(g));
+  const bool on_bricks = brick_grid(g) && g->shape.tx == kBrickTile.tx &&
+                         g->shape.ty == kBrickTile.ty;
+  info->ctas = on_bricks ? g->tiles_x * g->tiles_y * ((g->Nz + kBrickPlanes - 1) / kBrickPlanes)
+                         : sweep_ctas(g->R, g->shape, forward_mode(g));
   info->v_max = g->vmax;
   info->cfl_limit = g->cfl;
   info->launches = g_launches.load();

@@ -131,8 +131,10 @@ struct fd_grid_s {
   int sched_ctas = 0;              // CTAs of the wave-scheduled launch
   size_t sched_off = 0;            // byte offset of the items in g->sched
   int last_sched = 0;              // schedule of the last forward run (fd_grid_info)
-  fd::TileShape base_shape = {};   // tile of every run but tuned forward runs
-  bool auto_tile = false;          // no fd_set_tile: plain forward runs may be tuned
+  // tile of fd_set_tile or the default one: of decomposed runs, of schedules other
+  // than AUTO, and of grids with fd_set_tile (the others: use_shape)
+  fd::TileShape base_shape = {};
+  bool auto_tile = false;          // no fd_set_tile: AUTO takes bricks or wave tiles, and tunes
   bool tuned = false;              // tuned_shape / tuned_waves hold the tuner's pick
   fd::TileShape tuned_shape = {};
   fd::TileShape wave_shape = {};   // tile of runs on AUTO that are not tuned (0: not picked yet)
@@ -155,9 +157,11 @@ int radius_halo_x(int R);
 fd_status build_maps(fd_grid g);
 fd_status build_field_maps(fd_grid g, Fields& f);
 void set_shape(fd_grid g, TileShape t);
-// Puts the grid on the tile its next run uses: the tuned one for plain forward
-// runs of a tuned grid, else the base tile (rebuilding the tensor maps).
-fd_status use_shape(fd_grid g, bool plain_forward);
+// Puts the grid on the tile its next run uses (rebuilding the tensor maps).  Runs
+// of a whole grid (own_steps) under FD_SCHED_AUTO with no fd_set_tile: bricks where
+// brick_grid holds, else the tuned tile, else the wave tile.  All others: the base
+// tile.
+fd_status use_shape(fd_grid g, bool own_steps);
 // Times every compiled tile under both schedules on the grid's zeroed
 // wavefields (a few source-free steps each) and records the fastest for plain
 // forward runs; picks are cached per device and padded size.
