@@ -286,8 +286,8 @@ fd_status fd_set_tile(fd_grid grid, int32_t tile_x, int32_t tile_y, int32_t ctas
  *                    at least 400 steps: every compiled tile is timed under
  *                    both schedules for a few source-free steps on the
  *                    zeroed wavefields (cleared again before the run), twice,
- *                    and the fastest pair (column waves on the tile above
- *                    where they come within 2 %) serves all later runs of grids of
+ *                    and the fastest pair (column waves on 64 x 8 where
+ *                    they come within 1 %) serves all later runs of grids of
  *                    that padded size and kernel mode on that device
  *                    (fd_forward, fd_propagate and the adjoint; the pick is
  *                    cached per process; fd_grid_info shows the tile and

@@ -775,13 +775,17 @@ fd_status autotune_grid(fd_grid g) {
         pick = {t, g->tuned_waves};
       }
     }
-    // Pairs within a percent or two of the fastest are ranked by chance, and the
-    // adjoint's steps, which take the pick too, are not: of those, waves on
-    // wave_tile (296^3 SO 8, us a forward step / mean of a gradient's three: 64 x 8
-    // waves 79.6 / 103.2, shares 80.9 / 103.9, 32 x 16 waves 80.5 / 106.3)
-    const TileShape w = wave_tile(g);
+    // Pairs within a percent of the fastest are ranked by chance, and the adjoint's
+    // steps, which take the pick too, are not: of those, waves on 64 x 8.  us a step
+    // of the trial / of a whole gradient (three kinds of step), 64 x 8 waves against the
+    // best of the other near pairs: 296^3 SO 8 82.2 / 314.1, 82.9 / 323.6 (32 x 16 waves);
+    // 280 x 280 x 240 SO 12 94.7 / 348.0, 95.0 / 353.1 (32 x 16 waves); 296^3 SO 12
+    // 116.3 / 424.9, 116.3 / 431.9 (32 x 16 waves).  Beyond a percent the trial is right:
+    // 280 x 320 x 340 SO 8 107.5 / 388.2, 93.1 / 369.7 (32 x 16 waves); 240 x 280 x 280
+    // SO 16 106.8 / 373.5, 104.0 / 372.2 (32 x 16 shares).  Forward runs of nine sizes at
+    // SO 4 to 16 took the same time on either of two near pairs (within 0.3 %).
     for (int i = 0; i < kNumShapes; ++i)
-      if (kShapes[i].tx == w.tx && kShapes[i].ty == w.ty && best_of[2 * i + 1] <= 1.02f * best)
+      if (kShapes[i].tx == 16 && kShapes[i].ty == 8 && best_of[2 * i + 1] <= 1.01f * best)
         pick = {kShapes[i], true};
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
