@@ -155,7 +155,37 @@ __global__ void k_pad_coef(const float* __restrict__ phys, int R, int nx, int ny
   for (int j = 0; j < R; ++j) coef[j * ncell + dst] = phys[src + j];
 }
 
+// The TMA unit reads tensor maps through a proxy of its own and may hold what an
+// address held before its map was refreshed (another tile, or an adjoint segment's
+// checkpoint), so each refreshed map is fenced once, on every SM: the shared memory
+// of a block admits one per SM.  Everything later on the stream lies behind these
+// fences.  Fencing in the step kernels instead costs each CTA several fences: once per
+// run 15 us on 83 x 69 x 430 bricks, and in each launch 0.5 us a step on 84^3 and 5 us
+// on 149 x 128 x 103; maps passed as kernel parameters, which need no fence, cost 1 us a
+// step in launches outside graphs, as each brings them at an address no SM has seen.
+constexpr int kAcquireSmem = 120 * 1024;
+__global__ void k_acquire_maps(const unsigned char* maps, size_t stride, int groups, int per) {
+  for (int i = threadIdx.x; i < groups * per; i += blockDim.x)
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(
+                     maps + i / per * stride + size_t(i % per) * 128)
+                 : "memory");
+}
+
 }  // namespace
+
+cudaError_t acquire_maps(const void* maps, size_t stride, int groups, int per, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_acquire_maps, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kAcquireSmem);
+  if (e != cudaSuccess) return e;
+  k_acquire_maps<<<sms, 32, kAcquireSmem, s>>>(static_cast<const unsigned char*>(maps), stride,
+                                               groups, per);
+  count_launch();
+  return cudaGetLastError();
+}
 
 cudaError_t pad_coefficients(const float* phys, int R, int nx, int ny, int nz, int nbl, int Nx,
                              int Ny, int Nz, int pitch, size_t ncell, float* coef,

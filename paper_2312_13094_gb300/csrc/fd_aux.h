@@ -18,6 +18,11 @@ cudaError_t model_stats(const float* data, size_t n, int kind, float* vmin,
 cudaError_t model_to_A(const float* data, int kind, int nx, int ny, int nz, int nbl,
                        int Nx, int Ny, int Nz, int pitch, double dt2_h2, float* A,
                        cudaStream_t s);
+// Makes tensor maps in device memory that a host copy on `s` has written visible to
+// the TMA copies of the launches that follow on `s`: `groups` arrays of `per` maps,
+// `stride` bytes apart.
+cudaError_t acquire_maps(const void* maps, size_t stride, int groups, int per, cudaStream_t s);
+constexpr int kShotMaps = 6;  // maps at the start of a ShotDesc
 // Number of NaN/Inf values in x into *dcnt (device), without waiting for it.
 cudaError_t count_nonfinite_async(const float* x, size_t n, int* dcnt, cudaStream_t s);
 // The same, read into *hcnt (synchronises `s`).

@@ -190,6 +190,7 @@ fd_status upload_prepared(BatchWorkspace& ws, const Prepared& P, cudaStream_t s)
   cudaError_t e = ws.desc.ensure(P.host.size());
   if (e) return cuda_fail(e, "batch descriptor allocation");
   e = cudaMemcpyAsync(ws.desc.p, P.host.data(), P.host.size(), cudaMemcpyHostToDevice, s);
+  if (!e) e = acquire_maps(ws.desc.p, sizeof(ShotDesc), P.nshots, kShotMaps, s);
   if (!e) e = cudaStreamSynchronize(s);
   if (e) return cuda_fail(e, "batch descriptor upload");
   return FD_OK;
@@ -223,7 +224,6 @@ fd_status issue_steps(BatchWorkspace& ws, const Prepared& P, int R, const TileSh
     ov.rec_row = step;
     ov.spin_limit = P.spin_limit;
     ov.debug_skip_plane = -1;
-    ov.fresh = step == 0 ? P.nshots : 0;
     for (int j = 0; j < kMaxR + 2; ++j) ov.c[j] = P.c[j];
     if (P.waves) {
       const char* base = static_cast<const char*>(ws.desc.p);

@@ -64,10 +64,6 @@ __global__ void __launch_bounds__(BrickCfg<R, MODE>::NT, BrickCfg<R, MODE>::CTAS
   const StepArgs& a = shot->args;
   const int cur = ov.cur;
   pdl_trigger();
-  if (ov.fresh) {
-    acquire_maps(shot, 1);
-    __syncwarp();  // before the prefetch; before the copies, the barrier below
-  }
   if (tid < 3)  // the tensor maps, fetched while the step ahead still runs
     prefetch_map(tid == 0 ? &shot->halo[cur] : (tid == 1 ? &shot->tile[cur ^ 1] : &shot->A));
   if (tid == 0) {

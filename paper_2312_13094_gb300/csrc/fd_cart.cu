@@ -482,6 +482,7 @@ fd_status cart_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
   cudaError_t e = c->desc.ensure(host.size());
   if (e) return cuda_fail(e, "box descriptor allocation");
   e = cudaMemcpyAsync(c->desc.p, host.data(), host.size(), cudaMemcpyHostToDevice, g->stream);
+  if (!e) e = acquire_maps(c->desc.p, sizeof(ShotDesc), nbox, kShotMaps, g->stream);
   if (e) return cuda_fail(e, "box descriptor upload");
   if ((st = scatter(g, c))) return st;
 
@@ -564,7 +565,6 @@ fd_status cart_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
       ov.rec_row = t;
       ov.spin_limit = g->spin_limit;
       ov.debug_skip_plane = -1;
-      ov.fresh = t == 0 ? nbox : 0;
       ov.item_start = item_start;
       ov.items = items;
       launch_weights(g->c, R, ov.c);

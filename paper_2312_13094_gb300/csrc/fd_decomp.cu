@@ -309,6 +309,7 @@ fd_status decomp_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
   cudaError_t e = d->desc.ensure(host.size());
   if (e) return cuda_fail(e, "slab descriptor allocation");
   e = cudaMemcpyAsync(d->desc.p, host.data(), host.size(), cudaMemcpyHostToDevice, g->stream);
+  if (!e) e = acquire_maps(d->desc.p, kBlock, int(host.size() / kBlock), kShotMaps, g->stream);
   if (e) return cuda_fail(e, "slab descriptor upload");
   if ((st = scatter(g, d))) return st;
 
@@ -343,7 +344,6 @@ fd_status decomp_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
       ov.rec_row = t;
       ov.spin_limit = g->spin_limit;
       ov.debug_skip_plane = -1;
-      ov.fresh = t == 0 ? 1 : 0;
       launch_weights(g->c, R, ov.c);
       const ShotDesc* sd = reinterpret_cast<const ShotDesc*>(base + i * kBlock);
       const long long* pf = reinterpret_cast<const long long*>(base + i * kBlock + sizeof(ShotDesc));

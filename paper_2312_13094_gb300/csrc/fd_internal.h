@@ -111,8 +111,6 @@ struct StepOverride {
                              // centre weight's lo part
   const int32_t* item_start; // scheduled sweep: CTA c runs items [item_start[c],
   const WorkItem* items;     // item_start[c+1]); nullptr: equal contiguous shares
-  int fresh;                 // first launch since the tensor maps in device memory may
-                             // have changed: grids whose maps it acquires (else 0)
 };
 
 // Two-step (temporally blocked) pass, fd_tblock.cuh: what does not change
@@ -156,7 +154,6 @@ struct TbLaunch {
   float c[kMaxR + 2];  // as StepOverride::c
   const int32_t* item_start;
   const WorkItem* items;
-  int fresh;           // first pass of a run: acquire the tensor maps
 };
 
 // The weights of a uniform-stencil launch from the FP64 weights c[0..R]
@@ -173,13 +170,6 @@ inline void launch_weights(const double* c, int R, float* out) {
   t *= -6.0;
   out[0] = static_cast<float>(t);
   out[kMaxR + 1] = static_cast<float>(t - static_cast<double>(out[0]));
-}
-
-// Whether a kernel on `device` may address memory that cudaPointerGetAttributes
-// describes so: its own, or managed memory.  Memory of another device is left to
-// copies, which need no peer access.
-inline bool kernel_can_address(cudaMemoryType type, int owner, int device) {
-  return type == cudaMemoryTypeManaged || (type == cudaMemoryTypeDevice && owner == device);
 }
 
 struct TileShape {

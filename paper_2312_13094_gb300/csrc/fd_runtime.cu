@@ -853,13 +853,17 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
   e = g->desc.ensure(2 * sizeof(host));
   if (e) return cuda_fail(e, "descriptor allocation");
   char* dslot = static_cast<char*>(g->desc.p) + slot * sizeof(host);
-  // maps that the slot does not hold yet have to be acquired by the first step
+  // maps that the slot does not hold yet are acquired before the first step
+  static_assert(offsetof(ShotDesc, args) == kShotMaps * sizeof(CUtensorMap), "maps first");
   const char* maps = reinterpret_cast<const char*>(&host.d);
   std::vector<char>& sent = g->sent_maps[slot];
   const bool new_maps =
       sent.size() != offsetof(ShotDesc, args) || memcmp(sent.data(), maps, sent.size()) != 0;
   sent.clear();
   if (fd_status st = copy_in(g, dslot, &host, sizeof(host), "descriptor upload")) return st;
+  if (new_maps && (e = acquire_maps(dslot, 0, 1, kShotMaps, g->stream)))
+    return cuda_fail(e, "tensor maps");
+  sent.assign(maps, maps + offsetof(ShotDesc, args));
   const ShotDesc* dshot = reinterpret_cast<const ShotDesc*>(dslot);
   const long long* dprefix = reinterpret_cast<const long long*>(dslot + sizeof(ShotDesc));
 
@@ -907,7 +911,6 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
       ov.items = sched_ov.items;
       ov.spin_limit = g->spin_limit;
       ov.debug_skip_plane = (t == 0) ? g->debug_skip_plane : -1;
-      ov.fresh = t == 0 && (use_graph || new_maps) ? 1 : 0;  // (a graph serves later runs)
       launch_weights(g->c, g->R, ov.c);
       ov.inj_row = rs.inj_row0 + rs.inj_row_step * t;
       ov.rec_row = rs.rec_row0 + rs.rec_row_step * t;
@@ -944,7 +947,6 @@ fd_status run_steps(fd_grid g, const RunSpec& rs) {
     if (e) return cuda_fail(e, "graph launch");
     count_launch(rs.nsteps);
   }
-  sent.assign(maps, maps + offsetof(ShotDesc, args));
   F.cur = (cur0 + rs.nsteps) & 1;
   if (g->profiling) {
     cudaEventRecord(g->ev1, g->stream);

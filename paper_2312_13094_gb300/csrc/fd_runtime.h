@@ -67,6 +67,13 @@ struct GraphKey {
   float c[kMaxR + 2];
 };
 
+// Whether a kernel on `device` may address memory that cudaPointerGetAttributes
+// describes so: its own, or managed memory.  Memory of another device is left to
+// copies, which need no peer access.
+inline bool kernel_can_address(cudaMemoryType type, int owner, int device) {
+  return type == cudaMemoryTypeManaged || (type == cudaMemoryTypeDevice && owner == device);
+}
+
 struct Decomp;  // domain decomposition state of a grid (fd_decomp.cu)
 struct TbState;  // buffers of the two-step passes (fd_tblock.cu)
 struct Cart;     // boxes of a Cartesian decomposition (fd_cart.cu)

@@ -35,8 +35,6 @@
 //    error, waits (bounded) for its own copies still in flight, and returns.
 #pragma once
 
-#include <stddef.h>
-
 #include <climits>
 
 #include "fd_internal.h"
@@ -170,30 +168,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
     if (clock64() - t0 > limit) return false;
   }
   return true;
-}
-
-// Makes a tensor map that a host copy wrote to global memory visible to the
-// TMA unit, which reads maps through a proxy of its own and may hold what the
-// address held before.  (Maps in kernel parameters need no fence.)
-__device__ __forceinline__ void acquire_map(const CUtensorMap* map) {
-  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
-}
-
-// The maps of `nshots` grids, both parities, one by each thread; the copies follow
-// behind a CTA barrier.  The first launch that reads refreshed descriptors does
-// this in every CTA, and the run's later launches, ordered behind it, need not:
-// fencing each map in each launch costs 0.5 us a step of 84^3 bricks (5.6 us) and
-// 5 us one of 149 x 128 x 103 (12 us).  Passing the maps as kernel parameters, which
-// needs no fence, cost that gradient 1 us a step, as each launch then brings maps
-// at an address that no SM has seen.
-__device__ __forceinline__ void acquire_maps(const ShotDesc* shots, int nshots) {
-  static_assert(offsetof(ShotDesc, tile) == 2 * sizeof(CUtensorMap) &&
-                    offsetof(ShotDesc, A) == 4 * sizeof(CUtensorMap) &&
-                    offsetof(ShotDesc, C) == 5 * sizeof(CUtensorMap),
-                "halo[2], tile[2], A, C");
-  constexpr int kMaps = 6;  // C too: a later run with per-cell weights may find them unchanged
-  for (int i = threadIdx.x; i < kMaps * nshots; i += blockDim.x)
-    acquire_map(shots[i / kMaps].halo + i % kMaps);
 }
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map,
@@ -894,7 +868,6 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
   const long long hi = total * (blockIdx.x + 1) / gridDim.x;
   const int cur = ov.cur;
   pdl_trigger();
-  if (ov.fresh) acquire_maps(shots, ov.fresh);
   pdl_wait();
   int s = 0;
   for (long long pos = lo; pos < hi;) {
@@ -937,7 +910,6 @@ __global__ void __launch_bounds__(TX* TY, threads_per_sm(R, MODE) / (TX * TY))
   const int cur = ov.cur;
   const int i1 = ov.item_start[blockIdx.x + 1];
   pdl_trigger();
-  if (ov.fresh) acquire_maps(shots, ov.fresh);
   pdl_wait();
   for (int i = ov.item_start[blockIdx.x]; i < i1; ++i) {
     const WorkItem w = ov.items[i];

@@ -152,6 +152,8 @@ fd_status tblock_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
   cudaError_t e = t->desc.ensure(sizeof(TbDesc));
   if (e) return cuda_fail(e, "two-step descriptor");
   if ((st = copy_in(g, t->desc.p, &host, sizeof(host), "two-step descriptor"))) return st;
+  static_assert(offsetof(TbDesc, u) == 9 * sizeof(CUtensorMap), "nine maps");
+  if ((e = acquire_maps(t->desc.p, 0, 1, 9, g->stream))) return cuda_fail(e, "tensor maps");
 
   TbLaunch L;
   memset(&L, 0, sizeof(L));
@@ -172,7 +174,6 @@ fd_status tblock_propagate(fd_grid g, int n0, int nsteps, const fd_points* src,
     L.out2 = other + 1;
     L.inj_row = n0 + 2 * p;
     L.rec_row = 2 * p;
-    L.fresh = p == 0;
     count_launch();
     e = R == 2 ? launch_tblock_r<2>(dd, L, t->sched_ctas, g->stream)
                : launch_tblock_r<4>(dd, L, t->sched_ctas, g->stream);

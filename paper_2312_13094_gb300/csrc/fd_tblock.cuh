@@ -415,10 +415,6 @@ __global__ void __launch_bounds__(TbGeom<R>::NT, 1)
                   127u);
   __shared__ TbArgs a;
   if (threadIdx.x == 0) a = D->args;
-  static_assert(offsetof(TbDesc, ext) == 4 * sizeof(CUtensorMap) &&
-                    offsetof(TbDesc, extA) == 8 * sizeof(CUtensorMap),
-                "halo2[4], ext[4], extA");
-  if (L.fresh && threadIdx.x < 9) acquire_map(D->halo2 + threadIdx.x);
   __syncthreads();
   const int i1 = L.item_start[blockIdx.x + 1];
   for (int i = L.item_start[blockIdx.x]; i < i1; ++i) {

@@ -1,9 +1,9 @@
-// Host-side check of kernel_can_address (paper_2312_13094_gb300/csrc/fd_internal.h),
+// Host-side check of kernel_can_address (paper_2312_13094_gb300/csrc/fd_runtime.h),
 // built with g++ by tests/test_pointer_rule_host.py.  Prints one line per case:
 // memory type, owner, device, answer.
 #include <cstdio>
 
-#include "fd_internal.h"
+#include "fd_runtime.h"
 
 int main() {
   for (int type : {int(cudaMemoryTypeUnregistered), int(cudaMemoryTypeHost),
