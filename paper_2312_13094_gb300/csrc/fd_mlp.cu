@@ -537,14 +537,13 @@ __global__ void __launch_bounds__(NTHR, 2)
 
 // Sums of the blocks' gradients and losses.  Block b sums words [32 b, 32 b + 32)
 // of the gradient (8 threads side by side on a float4 each, 32 rows of blocks at
-// a time), the last block the losses.  Every sum is kept as hi + lo (Knuth's
+// a time, 5 rows ahead), the last block the losses.  Every sum is kept as hi + lo (Knuth's
 // two-sum, whose error term is exact), so that it adds one rounding whatever the
 // number of blocks.  Adding each block's sums to the words in global memory rounds
 // once per block: relative error of the gradient against FP64, mean of four to six
 // seeds, 1050 / 65 536 samples: 1.9e-7 / 2.5e-7 so, 0.95e-7 / 1.8e-7 with one block
-// of 128 samples per SM, 0.56e-7 / 0.55e-7 with this sum.  The call takes as long as
-// with the additions (33.7 and 81.8 us against 34.2 and 82.0): they cost the
-// training kernel what this launch costs behind it.  FP64 sums would be as exact;
+// of 128 samples per SM, 0.56e-7 / 0.55e-7 with this sum.  The call takes no longer than
+// with the additions: they cost the training kernel what this launch costs behind it.  FP64 sums would be as exact;
 // this GPU does about 2 of them per SM and clock.
 constexpr int SW = 8, SR = 32;  // float4 words and rows of a block
 __device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
@@ -571,25 +570,42 @@ __global__ void __launch_bounds__(SW* SR)
     }
     return;
   }
-  __shared__ float hi_of[SR][4 * SW], lo_of[SR][4 * SW];
+  __shared__ float hi_of[SR / 4][4 * SW], lo_of[SR / 4][4 * SW];
   const int q = tid % SW, row = tid / SW;
   const int w = (blockIdx.x * SW + q) * 4;
   float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
   if (w < NPARAM) {
-#pragma unroll 4
-    for (int b = row; b < blocks; b += SR) {
-      const float4 v = ld4(part + size_t(b) * NPARAM + w);
+    constexpr int kAhead = 5;  // loads in flight: 304 blocks are two rounds
+    for (int b = row; b < blocks; b += kAhead * SR) {
+      float4 v[kAhead];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) two_sum(hi[i], lo[i], at4(v, i));
+      for (int k = 0; k < kAhead; ++k)
+        v[k] = b + k * SR < blocks ? ld4(part + size_t(b + k * SR) * NPARAM + w)
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) two_sum(hi[i], lo[i], at4(v[k], i));
     }
   }
-  st4(&hi_of[row][4 * q], hi[0], hi[1], hi[2], hi[3]);
-  st4(&lo_of[row][4 * q], lo[0], lo[1], lo[2], lo[3]);
+  // the warp's four rows, then the warps
+#pragma unroll
+  for (int o = SW; o < 32; o *= 2)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float l = __shfl_xor_sync(0xffffffffu, lo[i], o);
+      two_sum(hi[i], lo[i], __shfl_xor_sync(0xffffffffu, hi[i], o));
+      lo[i] = __fadd_rn(lo[i], l);
+    }
+  if ((row & 3) == 0) {
+    st4(&hi_of[row / 4][4 * q], hi[0], hi[1], hi[2], hi[3]);
+    st4(&lo_of[row / 4][4 * q], lo[0], lo[1], lo[2], lo[3]);
+  }
   __syncthreads();
   if (tid >= 4 * SW || blockIdx.x * 4 * SW + tid >= NPARAM) return;
   float h = 0.f, l = 0.f;
 #pragma unroll
-  for (int r = 0; r < SR; ++r) {
+  for (int r = 0; r < SR / 4; ++r) {
     two_sum(h, l, hi_of[r][tid]);
     l = __fadd_rn(l, lo_of[r][tid]);
   }
@@ -833,8 +849,14 @@ static fd_status mlp_grad_device(fd_mlp net, int64_t n, const float* dsamples) {
     if (e) return cuda_fail(e, "kernel attribute");
     attr = true;
   }
-  // a small batch is spread one warp's samples per block
-  const int blocks = int(std::min<int64_t>(net->most_blocks, (n + NSUB - 1) / NSUB));
+  // One block per SM up to four chunks each: its eight warps take a chunk's units
+  // side by side, and every block is one more row to sum.  Two per SM beyond (us a
+  // call, one / two: 2009 samples 43.5 / 54.6, 8192 46.2 / 55.9, 20 000 58.2 / 68.4,
+  // 36 000 71.5 / 72.9, 65 536 93.2 / 92.4, 300 000 289 / 254).  A small batch is
+  // spread one warp's samples per block.
+  const int sms = net->most_blocks / 2;
+  const int most = n <= int64_t(4) * S * sms ? sms : 2 * sms;
+  const int blocks = int(std::min<int64_t>(most, (n + NSUB - 1) / NSUB));
   k_mlp_grad<<<blocks, NTHR, SM_GRAD * sizeof(float), net->stream>>>(
       net->p, dsamples, int(n), float(1.0 / double(n)), taylor_c(), net->part, net->lpart);
   count_launch(2);

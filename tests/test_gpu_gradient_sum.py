@@ -2,7 +2,7 @@
 rounding, whatever the number of blocks, and its order is fixed.
 
 B copies of the same eight samples make B blocks with the same partial sums
-(one block per eight samples up to two blocks per SM).  With B a power of two
+(one block per eight samples up to one block per SM).  With B a power of two
 the factor 1/n scales every term exactly, so the gradient of the B copies is
 that of the eight samples to the last bit; adding the blocks to an FP32 word
 one after the other rounds at every block that is no power of two."""
@@ -35,10 +35,10 @@ def samples(n, seed):
     return np.ascontiguousarray(np.concatenate([X, T, y[:, None], w[:, None]], 1), np.float32)
 
 
-@pytest.mark.parametrize("copies", [2, 16, 32, 64, 256])
+@pytest.mark.parametrize("copies", [2, 16, 32, 64, 128])
 def test_equal_blocks_add_up_exactly(learned, copies):
     import torch
-    if 2 * torch.cuda.get_device_properties(0).multi_processor_count < copies:
+    if torch.cuda.get_device_properties(0).multi_processor_count < copies:
         pytest.skip("fewer blocks than copies")
     net = learned.Network(mlp.init_params(11, scale_out=0.8).astype(np.float32))
     S = samples(8, 5)
@@ -62,10 +62,11 @@ def test_gradient_is_the_same_on_every_call(learned, n):
     net.close()
 
 
-@pytest.mark.parametrize("n", [8, 16, 17, 248, 256, 264, 2431, 2432, 2440])
+@pytest.mark.parametrize("n", [8, 16, 17, 248, 256, 264, 1216, 1224, 38912, 38913])
 def test_numbers_of_blocks_around_a_row_of_the_sum(learned, n):
-    """One block, two, and counts around the 32 rows that are summed side by
-    side, up to two blocks per SM and the first that take a second unit."""
+    """One block, two, counts around the 32 rows that are summed side by side, the
+    first that gives a block of 152 SMs a second unit, and the last with one block
+    per SM and the first with two."""
     th = mlp.init_params(13, scale_out=0.8).astype(np.float32)
     net = learned.Network(th)
     S = samples(n, n)

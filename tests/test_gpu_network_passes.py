@@ -1,7 +1,7 @@
 """Network kernels over more than one pass of the GPU: inference on rows and on
 a grid's cells (chunks of 128, four blocks per SM) where a block takes second
 and third chunks and the activation tile is used again, and the gradient where
-its staged samples are double-buffered (chunks of 64, two blocks per SM)."""
+its staged samples are double-buffered (chunks of 64)."""
 import numpy as np
 import pytest
 
@@ -48,8 +48,9 @@ def test_rows(learned, size):
 
 @pytest.mark.parametrize("chunks", [1.0, 1.5, 2.5, 3.25])
 def test_gradient(learned, chunks):
-    """Chunks of 64 per block: exactly one, one and a part, and enough that both
-    staging buffers are used again."""
+    """Chunks of 64, one block per SM up to four chunks and two beyond: two chunks of
+    one block, three, two and a part of two blocks, and three and a part, so that
+    both staging buffers are used again."""
     n = int(2 * sms() * 64 * chunks) + (3 if chunks > 1 else 0)
     rng = np.random.default_rng(n)
     S = np.concatenate([mlp.features(rng.uniform(1.5, 4.5, n), 20.0, 1.6, 12.0),
