@@ -481,8 +481,8 @@ fd_status propagate(fd_tti t, int n0, int nsteps, const fd_points* src, const fl
   qa.cols_y = (t->Ny + tti::kQY - 1) / tti::kQY;
   qa.cols = qa.cols_y * ((t->Nx + tti::kQX - 1) / tti::kQX);
   if (t->profiling) cudaEventRecord(t->ev0, t->stream);
-  // Launches may start before the one ahead has finished, up to SO 12 those of
-  // short steps.  us a step without / with it, at M padded cells:
+  // Launches of short steps may start before the one ahead has finished.  us a step
+  // without / with it, at M padded cells:
   //   SO 4   1.0 M 25.2 / 21.9   3.4 M  47.6 / 44.5    5.8 M  69.3 / 70.8   8.0 M   94 / 102
   //   SO 8   1.0 M 34.6 / 30.7   3.9 M  68.9 / 66.4    5.8 M  93.3 / 93.6  37.9 M  469 / 499
   //   SO 10  2.2 M 59.8 / 55.1   4.1 M  76.5 / 73.5   15.6 M 234.8 / 239.4 27.0 M  401 / 415
@@ -491,8 +491,9 @@ fd_status propagate(fd_tti t, int n0, int nsteps, const fd_points* src, const fl
   //   SO 16  1.0 M 54.5 / 48.8   4.1 M 108.1 / 103.6  19.7 M 433.2 / 428.9 63.8 M 1330 / 1326
   // CTAs that start where an earlier one ends break up the waves of neighbouring
   // columns, which share halos in L2; with the two CTAs per SM of SO 14 and 16 that
-  // costs less than the launch's latency at every size.
-  const bool early = t->R >= 7 || (long long)t->Nx * t->Ny * t->Nz <= 4000000LL;
+  // costs less than the launch's latency at every size up to those 64 M.
+  const bool early =
+      (long long)t->Nx * t->Ny * t->Nz <= (t->R >= 7 ? 64000000LL : 4000000LL);
   // sources of step `s` (-1: none) and receivers of the field it made, on u;
   // many of them in two launches of several blocks
   auto points = [&](int s, float2* u, bool first) -> cudaError_t {
