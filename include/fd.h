@@ -165,7 +165,8 @@ fd_status fd_backward(fd_grid grid, const fd_points* src, const float* wavelet,
  * are captured in a CUDA
  * graph when flags has FD_BATCH_GRAPH.  FD_BATCH_AUTOTUNE times the tile
  * candidates once per (space order, window sizes) and caches the choice.
- * All grids must be on the same device; the first grid's stream is used. */
+ * All grids must be on the same device; the first grid's stream is used, behind
+ * all that the other grids' streams hold when the call is made. */
 enum { FD_BATCH_GRAPH = 1, FD_BATCH_AUTOTUNE = 2 };
 typedef struct {
   fd_grid grid;
